@@ -201,13 +201,14 @@ size_t engine_resume_header_bytes(int P);
 // descriptors after those of the groups before it.
 int engine_capture(ProblemDev *pds, const int *sizes, int groups, const ccs_params &prm, char *ws,
                    ccs_result *dev_out, cudaGraphExec_t *exec);
-// The expander's construction in two enqueued parts (ccs_setup.cu), for
-// callers that batch the read-back of the largest row degree.
+// The expander's construction (ccs_setup.cu): all of it enqueued, then what
+// the largest row degree, read back by the caller, may still ask for.
 int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
                          int64_t *csr_ptr, int32_t *csr_cols, void *ws, cudaStream_t s,
                          int **max_deg_dev);
-int expander_sort_rows(int32_t m, int64_t *csr_ptr, int32_t *csr_cols, int host_max,
-                       cudaStream_t s);
+int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
+                    int64_t *csr_ptr, int32_t *csr_cols, void *ws, int host_max, cudaStream_t s,
+                    bool *again);
 
 int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
                   char *hdr, cudaStream_t s);

@@ -184,9 +184,8 @@ static size_t seeded_layout(int32_t n, int32_t m, int32_t d, int32_t max_iter, i
 
 // Seeded requests just admitted (indices `todo` of inflight): upload each y,
 // draw each A from its seed into the pool -- every request's construction
-// enqueued first, then one wait for all their largest row degrees, then the
-// row sorts -- so the worker waits on the stream once per admission, not
-// once per request.  rcs[q] receives each request's status.
+// enqueued first, then one wait for all their largest row degrees -- so the
+// worker waits on the stream once per admission, not once per request.  rcs[q] receives each request's status.
 static void prepare_seeded(ccs_server *S, const std::vector<int> &todo, std::vector<int> &rcs) {
     const int Q = (int)todo.size();
     rcs.assign(Q, CCS_OK);
@@ -225,9 +224,12 @@ static void prepare_seeded(ccs_server *S, const std::vector<int> &todo, std::vec
     for (int q = 0; q < Q; ++q) {
         if (rcs[q]) continue;
         Request &R = S->inflight[todo[q]];
-        rcs[q] = expander_sort_rows(R.host.m, const_cast<int64_t *>(R.prob.csr_ptr),
-                                    const_cast<int32_t *>(R.prob.csr_cols), S->host_max[q],
-                                    S->stream);
+        bool again = false;
+        rcs[q] = expander_finish(R.host.n, R.host.m, R.host.d, R.host.a_seed,
+                                 const_cast<int32_t *>(R.prob.csc_rows),
+                                 const_cast<int64_t *>(R.prob.csr_ptr),
+                                 const_cast<int32_t *>(R.prob.csr_cols), gen[q], S->host_max[q],
+                                 S->stream, &again);
         if (!rcs[q]) R.prepared = true;
     }
 }

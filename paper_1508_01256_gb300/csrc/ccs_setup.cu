@@ -4,6 +4,8 @@
 // independently, each column's support uniform over the C(m, d) subsets of
 // size d.  Every column owns a counter-based SplitMix64 stream, so a column
 // is one thread's work and the matrix depends only on (n, m, d, seed).
+#include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 
@@ -27,59 +29,103 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t &state) {
 }
 
 // Lemire's bounded draw (ACM TOMACS 2019): high word of x * range, redrawing
-// while the low word is below 2^64 mod range.
+// while the low word is below 2^64 mod range.  The 96-bit product is formed
+// from two 32 x 32-bit ones (range has 32 bits).
 __device__ __forceinline__ uint32_t draw_below(uint64_t &state, uint32_t range) {
     uint64_t x = splitmix64(state);
-    uint64_t lo = x * (uint64_t)range;
-    uint64_t hi = __umul64hi(x, (uint64_t)range);
+    uint64_t p0 = (x & 0xffffffffull) * range, p1 = (x >> 32) * range + (p0 >> 32);
+    uint64_t lo = (p1 << 32) | (p0 & 0xffffffffull);
     if (lo < range) {
         const uint64_t floor_mod = (0ull - (uint64_t)range) % (uint64_t)range;
         while (lo < floor_mod) {
             x = splitmix64(state);
-            lo = x * (uint64_t)range;
-            hi = __umul64hi(x, (uint64_t)range);
+            p0 = (x & 0xffffffffull) * range;
+            p1 = (x >> 32) * range + (p0 >> 32);
+            lo = (p1 << 32) | (p0 & 0xffffffffull);
         }
     }
-    return (uint32_t)hi;
+    return (uint32_t)(p1 >> 32);
 }
 
-// One thread per column: d distinct rows, sorted ascending.
-__global__ void k_generate_columns(int n, int m, int d, uint64_t seed, int32_t *csc_rows) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
+// Column j's D distinct rows, ascending, in registers.
+template <int D>
+__device__ __forceinline__ void draw_column(int j, int m, uint64_t seed, int32_t (&rows)[D]) {
     uint64_t state = seed + (uint64_t)(j + 1) * 0xd1b54a32d192ed03ull;
-    int32_t rows[kMaxD];
-    int got = 0;
-    while (got < d) {
-        const int32_t row = (int32_t)draw_below(state, (uint32_t)m);
-        bool seen = false;
-        for (int t = 0; t < got; ++t) seen |= (rows[t] == row);
-        if (!seen) rows[got++] = row;
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+        bool seen;
+        do {
+            rows[t] = (int32_t)draw_below(state, (uint32_t)m);
+            seen = false;
+#pragma unroll
+            for (int q = 0; q < t; ++q) seen |= (rows[q] == rows[t]);
+        } while (seen);
     }
-    for (int a = 1; a < d; ++a) {
-        const int32_t v = rows[a];
-        int b = a - 1;
-        while (b >= 0 && rows[b] > v) {
-            rows[b + 1] = rows[b];
-            --b;
+    // compare-exchange rounds of neighbours: D of them sort D values
+#pragma unroll
+    for (int round = 0; round < D; ++round)
+#pragma unroll
+        for (int q = round & 1; q + 1 < D; q += 2) {
+            const int32_t lo = min(rows[q], rows[q + 1]), hi = max(rows[q], rows[q + 1]);
+            rows[q] = lo;
+            rows[q + 1] = hi;
         }
-        rows[b + 1] = v;
+}
+
+// A block's columns (their rows laid out one column after another in shared
+// memory) to the CSC array by 16-byte stores: `ints` of them from dst, which
+// is 16-byte aligned.
+__device__ __forceinline__ void store_columns(const int32_t *stage, int32_t *dst, int ints) {
+    for (int q = threadIdx.x; q < ints / 4; q += blockDim.x)
+        reinterpret_cast<int4 *>(dst)[q] = reinterpret_cast<const int4 *>(stage)[q];
+    for (int q = (ints & ~3) + threadIdx.x; q < ints; q += blockDim.x) dst[q] = stage[q];
+}
+
+// One thread a column, and one atomic add per entry counts its row.  With shift > 0 the add's result, the
+// entry's rank in its row, rides in the bits of the row index above `shift`
+// (k_place_ranked takes it out again), so that placing the transpose needs
+// no second round of atomics.
+//
+// Bound by the 64-bit integer work of the draws (~25 instructions each) and
+// the atomics; the entries go through shared memory so that the stores are
+// whole lines instead of 4 d-byte pieces.
+constexpr int kGenBlock = 256;
+template <int D>
+__global__ void __launch_bounds__(kGenBlock)
+k_generate_columns(int n, int m, uint64_t seed, int shift, int32_t *csc_rows, int32_t *deg) {
+    __shared__ __align__(16) int32_t stage[kGenBlock * D];
+    const int j0 = blockIdx.x * kGenBlock, j = j0 + threadIdx.x;
+    if (j < n) {
+        int32_t rows[D];
+        draw_column<D>(j, m, seed, rows);
+        if (shift) {
+            int rank[D];
+#pragma unroll
+            for (int t = 0; t < D; ++t) rank[t] = atomicAdd(deg + rows[t], 1);
+#pragma unroll
+            for (int t = 0; t < D; ++t)
+                stage[threadIdx.x * D + t] = rows[t] | (int32_t)((uint32_t)rank[t] << shift);
+        } else {
+#pragma unroll
+            for (int t = 0; t < D; ++t) {
+                atomicAdd(deg + rows[t], 1);
+                stage[threadIdx.x * D + t] = rows[t];
+            }
+        }
     }
-    int32_t *out = csc_rows + (size_t)j * d;
-    for (int t = 0; t < d; ++t) out[t] = rows[t];
+    __syncthreads();
+    store_columns(stage, csc_rows + (size_t)j0 * D, min(kGenBlock, n - j0) * D);
 }
 
 // ---------------------------------------------------------------------------
-// CSR transpose: count -> scan -> scatter -> sort each row
+// CSR transpose: row degrees -> scan -> place -> sort each row
 // ---------------------------------------------------------------------------
-
-__global__ void k_count_rows(long long edges, const int32_t *csc_rows, int32_t *deg) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < edges;
-         e += (long long)gridDim.x * blockDim.x)
-        atomicAdd(&deg[csc_rows[e]], 1);
-}
 
 constexpr int kScanBlock = 1024;
+constexpr int kWarpSortCap = 512;   // longest row a warp sorts in registers
+constexpr int kGroupEntries = 36864;  // entries a group of rows has at most, on average
+constexpr int kMaxGroups = 8192;      // counted on chip
+constexpr int kMaxGroupRowBits = 12;
 
 // Per block of kScanBlock rows: inclusive prefix of deg into ptr[1 + i],
 // block total into sums[block], largest degree into *max_deg.
@@ -116,47 +162,50 @@ k_scan_local(int m, const int32_t *deg, int64_t *ptr, int64_t *sums, int *max_de
     if (threadIdx.x == kScanBlock - 1) sums[blockIdx.x] = inc;
 }
 
-// Exclusive scan of the block totals, one block, sequential over chunks.
-__global__ void __launch_bounds__(1024) k_scan_sums(int nblocks, int64_t *sums) {
-    __shared__ long long warp_tot[32];
-    __shared__ long long carry;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) carry = 0;
+// ptr += the totals of the blocks before (each block sums them itself).
+__global__ void __launch_bounds__(kScanBlock) k_scan_add(int m, int64_t *ptr, const int64_t *sums) {
+    __shared__ unsigned long long before;
+    const int i = blockIdx.x * kScanBlock + threadIdx.x;
+    if (threadIdx.x == 0) before = 0;
     __syncthreads();
-    for (int base = 0; base < nblocks; base += 1024) {
-        const int i = base + threadIdx.x;
-        long long v = (i < nblocks) ? sums[i] : 0;
-        long long inc = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            long long t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += t;
-        }
-        if (lane == 31) warp_tot[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            long long w = warp_tot[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                long long t = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += t;
-            }
-            warp_tot[lane] = w;
-        }
-        __syncthreads();
-        if (warp > 0) inc += warp_tot[warp - 1];
-        const long long c = carry;
-        if (i < nblocks) sums[i] = c + inc - v;  // exclusive
-        __syncthreads();
-        if (threadIdx.x == 1023) carry = c + inc;
-        __syncthreads();
-    }
+    long long v = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanBlock) v += sums[b];
+    v = warp_sum_ll(v);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&before, (unsigned long long)v);
+    __syncthreads();
+    if (i == 0) ptr[0] = 0;
+    if (i < m) ptr[i + 1] += (long long)before;
 }
 
-__global__ void k_scan_add(int m, int64_t *ptr, const int64_t *sums) {
-    const int i = blockIdx.x * kScanBlock + threadIdx.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ptr[0] = 0;
-    if (i < m) ptr[i + 1] += sums[blockIdx.x];
+// Entries of a k_generate_columns that packed their ranks: each goes to its
+// place in its row, and the CSC array gets the plain row index back.  A
+// thread takes four entries (one 16-byte load and store of the CSC).
+template <int D>
+__global__ void k_place_ranked(long long edges, int shift, int32_t *csc_rows, const int64_t *ptr,
+                               int32_t *csr_cols) {
+    const uint32_t mask = (1u << shift) - 1u;
+    const long long quads = edges / 4;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < quads; q += step) {
+        int4 v = reinterpret_cast<int4 *>(csc_rows)[q];
+        uint32_t e[4] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z, (uint32_t)v.w};
+        int64_t at[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) at[t] = __ldg(ptr + (e[t] & mask)) + (e[t] >> shift);
+        v.x = (int)(e[0] & mask);
+        v.y = (int)(e[1] & mask);
+        v.z = (int)(e[2] & mask);
+        v.w = (int)(e[3] & mask);
+        reinterpret_cast<int4 *>(csc_rows)[q] = v;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) csr_cols[at[t]] = (int32_t)((uint32_t)(4 * q + t) / D);
+    }
+    const long long r = quads * 4 + blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (r < edges) {
+        const uint32_t e = (uint32_t)csc_rows[r];
+        csc_rows[r] = (int32_t)(e & mask);
+        csr_cols[__ldg(ptr + (e & mask)) + (e >> shift)] = (int32_t)((uint32_t)r / D);
+    }
 }
 
 __global__ void k_scatter_cols(int n, int d, const int32_t *csc_rows, const int64_t *ptr,
@@ -170,45 +219,78 @@ __global__ void k_scatter_cols(int n, int d, const int32_t *csc_rows, const int6
     }
 }
 
-// One block per row: bitonic sort of the row's columns in shared memory
-// (padded with INT_MAX to `cap`, a power of two).
-__global__ void k_sort_rows(int m, int cap, const int64_t *ptr, int32_t *csr_cols) {
-    extern __shared__ int32_t buf[];
+// One block per row: bucket sort of the row's columns in shared memory.  The
+// columns of a row are uniform over [0, n), so buckets of equal width
+// (2^shift columns, `buckets` of them cover n) hold a few each (~8), and a
+// thread sorts a bucket by insertion.  Any other distribution is sorted too,
+// only slower.  Rows longer than `cap` are left alone.
+//
+// The row is read twice (the second time from cache) and written once; the
+// compare-exchange network it replaces took log2(len)^2 / 2 passes over
+// shared memory (12.5 ms at n = 2^24, m = 16777, d = 9).
+constexpr int kSortBlock = 512;
+__global__ void __launch_bounds__(kSortBlock)
+k_sort_rows(int m, int cap, int shift, int buckets, const int64_t *ptr, int32_t *csr_cols) {
+    extern __shared__ int32_t sm[];
+    int32_t *end = sm, *buf = sm + buckets;  // buckets, cap
+    __shared__ int warp_tot[kSortBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = blockIdx.x; i < m; i += gridDim.x) {
         const int64_t b = ptr[i];
         const int len = (int)(ptr[i + 1] - b);
-        if (len > 1) {
-            int size = 2;
-            while (size < len) size <<= 1;
-            for (int t = threadIdx.x; t < size; t += blockDim.x)
-                buf[t] = t < len ? csr_cols[b + t] : 0x7fffffff;
-            __syncthreads();
-            for (int k = 2; k <= size; k <<= 1) {
-                for (int jj = k >> 1; jj > 0; jj >>= 1) {
-                    for (int t = threadIdx.x; t < size; t += blockDim.x) {
-                        const int p = t ^ jj;
-                        if (p > t) {
-                            const bool up = (t & k) == 0;
-                            const int32_t a = buf[t], c = buf[p];
-                            if ((a > c) == up) {
-                                buf[t] = c;
-                                buf[p] = a;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
-            for (int t = threadIdx.x; t < len; t += blockDim.x) csr_cols[b + t] = buf[t];
-            __syncthreads();
+        if (len <= 1 || len > cap) continue;
+        for (int q = threadIdx.x; q < buckets; q += kSortBlock) end[q] = 0;
+        __syncthreads();
+        for (int t = threadIdx.x; t < len; t += kSortBlock)
+            atomicAdd(end + (csr_cols[b + t] >> shift), 1);
+        __syncthreads();
+        // exclusive prefix of the counts: a run of buckets a thread
+        const int per = (buckets + kSortBlock - 1) / kSortBlock;
+        const int q0 = min(buckets, (int)threadIdx.x * per), q1 = min(buckets, q0 + per);
+        int sum = 0;
+        for (int q = q0; q < q1; ++q) sum += end[q];
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
         }
+        if (lane == 31) warp_tot[warp] = inc;
+        __syncthreads();
+        int run = inc - sum;
+        for (int w = 0; w < warp; ++w) run += warp_tot[w];
+        for (int q = q0; q < q1; ++q) {
+            const int c = end[q];
+            end[q] = run;
+            run += c;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < len; t += kSortBlock) {
+            const int32_t c = csr_cols[b + t];
+            buf[atomicAdd(end + (c >> shift), 1)] = c;
+        }
+        __syncthreads();  // end[q] is now bucket q's end
+        for (int q = threadIdx.x; q < buckets; q += kSortBlock) {
+            const int lo = q ? end[q - 1] : 0, hi = end[q];
+            for (int t = lo + 1; t < hi; ++t) {
+                const int32_t c = buf[t];
+                int u = t - 1;
+                while (u >= lo && buf[u] > c) {
+                    buf[u + 1] = buf[u];
+                    --u;
+                }
+                buf[u + 1] = c;
+            }
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < len; t += kSortBlock) csr_cols[b + t] = buf[t];
+        __syncthreads();
     }
-    (void)cap;
 }
 
 // Rows of at most 32 E columns: one warp a row, the row in registers (E per
 // lane, element lane * E + e), bitonic sort by register exchanges and warp
-// shuffles: no shared memory and no block barriers.
+// shuffles: no shared memory and no block barriers.  Longer rows are left alone.
 template <int E>
 __global__ void k_sort_rows_warp(int m, const int64_t *ptr, int32_t *csr_cols) {
     constexpr int kCap = 32 * E;
@@ -218,7 +300,7 @@ __global__ void k_sort_rows_warp(int m, const int64_t *ptr, int32_t *csr_cols) {
     for (long long i = w0; i < m; i += nw) {
         const int64_t b = ptr[i];
         const int len = (int)(ptr[i + 1] - b);
-        if (len <= 1) continue;
+        if (len <= 1 || len > kCap) continue;
         int32_t v[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -259,6 +341,238 @@ __global__ void k_sort_rows_warp(int m, const int64_t *ptr, int32_t *csr_cols) {
             const int idx = lane * E + e;
             if (idx < len) csr_cols[b + idx] = v[e];
         }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Grouped construction: draw -> partition by group of rows -> sort each group
+// ---------------------------------------------------------------------------
+//
+// Rows are taken in groups of 2^row_bits whose entries fit one CTA's shared
+// memory.  The columns are drawn and the groups' sizes counted on chip; a
+// second pass deals the entries out to their groups' parts of csr_cols, a
+// block's entries ordered by group on chip first so that they leave as runs;
+// then a CTA a group sorts its entries by (row, column), which also gives
+// the row offsets.  An entry on its way is one word, its row in the group
+// above its column, so nothing beyond csr_cols is needed.
+//
+// What it replaces took two rounds of global atomics per entry, a scattered
+// 4-byte store (about 130 G/s each, whatever their size) and a sort of
+// log2(len)^2 / 2 passes: 18.2 ms at n = 2^24, m = 16777, d = 9, against
+// three passes over the entries.
+
+// Columns of this block's turn, their CSC entries stored, the entries per
+// group added to size[0, groups).
+constexpr int kDrawBlock = 512;
+template <int D>
+__global__ void __launch_bounds__(kDrawBlock)
+k_draw_columns(int n, int m, uint64_t seed, int row_bits, int groups, int32_t *csc_rows,
+               int32_t *size) {
+    extern __shared__ __align__(16) int32_t sm[];
+    int32_t *stage = sm, *cnt = sm + kDrawBlock * D;  // kDrawBlock D, groups
+    for (int g = threadIdx.x; g < groups; g += kDrawBlock) cnt[g] = 0;
+    __syncthreads();
+    for (long long j0 = (long long)blockIdx.x * kDrawBlock; j0 < n;
+         j0 += (long long)gridDim.x * kDrawBlock) {
+        const long long j = j0 + threadIdx.x;
+        if (j < n) {
+            int32_t rows[D];
+            draw_column<D>((int)j, m, seed, rows);
+#pragma unroll
+            for (int t = 0; t < D; ++t) {
+                stage[threadIdx.x * D + t] = rows[t];
+                atomicAdd(cnt + (rows[t] >> row_bits), 1);
+            }
+        }
+        __syncthreads();
+        store_columns(stage, csc_rows + (size_t)j0 * D, (int)min((long long)kDrawBlock, n - j0) * D);
+        __syncthreads();
+    }
+    for (int g = threadIdx.x; g < groups; g += kDrawBlock)
+        if (cnt[g]) atomicAdd(size + g, cnt[g]);
+}
+
+// Exclusive prefix of one int per thread over the block (kDealBlock threads).
+constexpr int kDealBlock = 1024;
+__device__ __forceinline__ int deal_scan(int v) {
+    __shared__ int warp_tot[kDealBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    __syncthreads();  // earlier users of warp_tot are done
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    const int w = warp_tot[lane];
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0);
+    return before + inc - v;
+}
+
+// Group sizes -> first entries (one block).
+__global__ void __launch_bounds__(kDealBlock) k_scan_groups(int groups, int32_t *size) {
+    const int per = (groups + kDealBlock - 1) / kDealBlock;
+    const int g0 = min(groups, (int)threadIdx.x * per), g1 = min(groups, g0 + per);
+    int sum = 0;
+    for (int g = g0; g < g1; ++g) sum += size[g];
+    int run = deal_scan(sum);
+    for (int g = g0; g < g1; ++g) {
+        const int c = size[g];
+        size[g] = run;
+        run += c;
+    }
+}
+
+// Entries to their groups.  A block takes kDealPer entries a thread at a
+// time, ranks them by group with shared-memory atomics, reserves each
+// group's run (next[g], which starts as the group's first entry and ends as
+// its last), lays the entries out by group on chip and stores them in that
+// order: consecutive threads store consecutive words of a run.
+constexpr int kDealPer = 24;
+template <int D>
+__global__ void __launch_bounds__(kDealBlock)
+k_deal_entries(uint32_t edges, int row_bits, int col_bits, int groups, int per,
+               const int32_t *csc_rows, int32_t *next, int32_t *csr_cols) {
+    extern __shared__ __align__(16) int32_t sm[];
+    int32_t *cnt = sm, *to = sm + groups;                     // groups each
+    uint32_t *val = reinterpret_cast<uint32_t *>(to + groups);  // kDealBlock per
+    uint16_t *grp = reinterpret_cast<uint16_t *>(val + kDealBlock * per);
+    const uint32_t row_mask = (1u << row_bits) - 1u;
+    const uint32_t turn = (uint32_t)(kDealBlock * per);
+    for (uint64_t e0 = (uint64_t)blockIdx.x * turn; e0 < edges; e0 += (uint64_t)gridDim.x * turn) {
+        const uint32_t len = (uint32_t)min((uint64_t)turn, edges - e0);
+        for (int g = threadIdx.x; g < groups; g += kDealBlock) cnt[g] = 0;
+        __syncthreads();
+        int32_t row[kDealPer];
+        uint16_t rank[kDealPer];
+#pragma unroll
+        for (int k = 0; k < kDealPer; ++k) {
+            const uint32_t q = threadIdx.x + k * kDealBlock;
+            row[k] = (k < per && q < len) ? __ldcs(csc_rows + e0 + q) : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < kDealPer; ++k)
+            if (row[k] >= 0) rank[k] = (uint16_t)atomicAdd(cnt + (row[k] >> row_bits), 1);
+        __syncthreads();
+        const int gper = (groups + kDealBlock - 1) / kDealBlock;
+        const int g0 = min(groups, (int)threadIdx.x * gper), g1 = min(groups, g0 + gper);
+        int sum = 0;
+        for (int g = g0; g < g1; ++g) {
+            const int c = cnt[g];
+            to[g] = c ? atomicAdd(next + g, c) : 0;
+            sum += c;
+        }
+        int run = deal_scan(sum);
+        for (int g = g0; g < g1; ++g) {
+            const int c = cnt[g];
+            cnt[g] = run;   // where the group starts on chip
+            to[g] -= run;   // and how far its run is from there
+            run += c;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kDealPer; ++k)
+            if (row[k] >= 0) {
+                const int g = row[k] >> row_bits, p = cnt[g] + rank[k];
+                const uint32_t e = (uint32_t)e0 + threadIdx.x + k * kDealBlock;
+                val[p] = (e / D) | (((uint32_t)row[k] & row_mask) << col_bits);
+                grp[p] = (uint16_t)g;
+            }
+        __syncthreads();
+        for (uint32_t p = threadIdx.x; p < len; p += kDealBlock)
+            csr_cols[to[grp[p]] + (int)p] = (int32_t)val[p];
+        __syncthreads();
+    }
+}
+
+// One CTA a group: its entries sorted by (row, column), the rows' offsets,
+// and the largest degree.  Equal-width buckets of the packed word hold a few
+// entries each (columns are uniform), and a thread sorts a bucket by
+// insertion; any distribution is sorted, only slower.  The entries are read
+// twice, the second time from cache.  end[g] is the group's last entry; a
+// group of more than `cap` entries sets *max_deg to INT_MAX.
+constexpr int kGroupBlock = 1024;
+__global__ void __launch_bounds__(kGroupBlock)
+k_sort_groups(int m, int groups, int row_bits, int col_bits, int shift, int buckets, int cap,
+              const int32_t *end, int64_t *csr_ptr, int32_t *csr_cols, int *max_deg) {
+    extern __shared__ __align__(16) int32_t sm[];
+    int32_t *top = sm;                                       // buckets
+    int32_t *row_end = sm + buckets;                         // 2^row_bits
+    uint32_t *buf = reinterpret_cast<uint32_t *>(row_end + (1 << row_bits));  // cap
+    const uint32_t col_mask = (1u << col_bits) - 1u;
+    for (int g = blockIdx.x; g < groups; g += gridDim.x) {
+        const int b = g ? end[g - 1] : 0, len = end[g] - b;
+        const int r0 = g << row_bits, rows = min(1 << row_bits, m - r0);
+        if (len > cap) {
+            if (threadIdx.x == 0) atomicMax(max_deg, 0x7fffffff);
+            continue;
+        }
+        uint32_t *src = reinterpret_cast<uint32_t *>(csr_cols) + b;
+        __syncthreads();  // the previous group's readers are done
+        for (int q = threadIdx.x; q < buckets; q += kGroupBlock) top[q] = 0;
+        for (int r = threadIdx.x; r < rows; r += kGroupBlock) row_end[r] = 0;
+        __syncthreads();
+#pragma unroll 4
+        for (int t = threadIdx.x; t < len; t += kGroupBlock) atomicAdd(top + (src[t] >> shift), 1);
+        __syncthreads();
+        const int per = (buckets + kGroupBlock - 1) / kGroupBlock;
+        const int q0 = min(buckets, (int)threadIdx.x * per), q1 = min(buckets, q0 + per);
+        int sum = 0;
+        for (int q = q0; q < q1; ++q) sum += top[q];
+        int run = deal_scan(sum);
+        for (int q = q0; q < q1; ++q) {
+            const int c = top[q];
+            top[q] = run;
+            run += c;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int t = threadIdx.x; t < len; t += kGroupBlock) {
+            const uint32_t v = src[t];
+            buf[atomicAdd(top + (v >> shift), 1)] = v;
+        }
+        __syncthreads();  // top[q] is now bucket q's end
+        for (int q = threadIdx.x; q < buckets; q += kGroupBlock) {
+            const int lo = q ? top[q - 1] : 0, hi = top[q];
+            for (int t = lo + 1; t < hi; ++t) {
+                const uint32_t v = buf[t];
+                int u = t - 1;
+                while (u >= lo && buf[u] > v) {
+                    buf[u + 1] = buf[u];
+                    --u;
+                }
+                buf[u + 1] = v;
+            }
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < len; t += kGroupBlock) {
+            const uint32_t v = buf[t], r = v >> col_bits;
+            src[t] = v & col_mask;
+            const uint32_t after = t + 1 < len ? buf[t + 1] >> col_bits : (uint32_t)rows;
+            if (after != r) row_end[r] = t + 1;  // the row's last entry
+        }
+        __syncthreads();
+        // rows without entries end where the row before does
+        int mx = 0;
+        const int rper = (rows + kGroupBlock - 1) / kGroupBlock;
+        const int a0 = min(rows, (int)threadIdx.x * rper), a1 = min(rows, a0 + rper);
+        int last = 0;
+        for (int r = a0 - 1; r >= 0 && a0 < a1; --r)
+            if (row_end[r]) {
+                last = row_end[r];
+                break;
+            }
+        for (int r = a0; r < a1; ++r) {
+            const int e = row_end[r] ? row_end[r] : last;
+            csr_ptr[(int64_t)r0 + r + 1] = (int64_t)b + e;
+            mx = max(mx, e - last);
+            last = e;
+        }
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((threadIdx.x & 31) == 0 && mx) atomicMax(max_deg, mx);
+        if (g == 0 && threadIdx.x == 0) csr_ptr[0] = 0;
     }
 }
 
@@ -451,75 +765,232 @@ size_t ccs_workspace_size(int32_t op, int32_t n, int32_t m, int32_t d) {
 
 namespace ccs {
 
-// First part of the expander's construction, all enqueued on `s`: the
-// columns, the row degrees and their prefix (csr_ptr), the CSR scatter.
-// *max_deg_dev receives the device address of the largest row degree, which
-// sizes the row sort (expander_sort_rows).  Arguments already checked.
-int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
-                         int64_t *csr_ptr, int32_t *csr_cols, void *ws, cudaStream_t s,
-                         int **max_deg_dev) {
-    char *base = static_cast<char *>(ws);
-    int32_t *deg = reinterpret_cast<int32_t *>(base);
-    const int nblocks = (m + kScanBlock - 1) / kScanBlock;
-    int64_t *sums = reinterpret_cast<int64_t *>(base + align_up((size_t)m * 4, 256));
-    int *max_deg = reinterpret_cast<int *>(base + align_up((size_t)m * 4, 256) +
-                                           align_up((size_t)nblocks * 8, 256));
-    const long long edges = (long long)n * d;
+// How (n, m, d) is drawn and transposed.
+struct ExpanderPlan {
+    int sms;
+    int groups;             // > 0: grouped construction
+    int row_bits, col_bits;
+    int group_cap;          // entries a group is not expected to pass
+    int buckets, shift;     // of the group sort
+    int deal_per;           // entries a thread of the deal takes at a time
+    size_t draw_smem, deal_smem, sort_smem;
+    // otherwise:
+    int rank_shift;         // > 0: ranks ride above this bit of the row indices
+    int cap;                // row length the sort is sized for
+};
 
-    k_generate_columns<<<(n + 255) / 256, 256, 0, s>>>(n, m, d, seed, csc_rows);
-    CCS_CUDA_TRY(cudaGetLastError());
-    CCS_CUDA_TRY(cudaMemsetAsync(deg, 0, (size_t)m * 4, s));
-    CCS_CUDA_TRY(cudaMemsetAsync(max_deg, 0, sizeof(int), s));
-    k_count_rows<<<grid_for(edges, 256), 256, 0, s>>>(edges, csc_rows, deg);
-    k_scan_local<<<nblocks, kScanBlock, 0, s>>>(m, deg, csr_ptr, sums, max_deg);
-    k_scan_sums<<<1, 1024, 0, s>>>(nblocks, sums);
-    k_scan_add<<<nblocks, kScanBlock, 0, s>>>(m, csr_ptr, sums);
-    CCS_CUDA_TRY(cudaGetLastError());
-    CCS_CUDA_TRY(cudaMemsetAsync(deg, 0, (size_t)m * 4, s));
-    k_scatter_cols<<<grid_for(edges, 256), 256, 0, s>>>(n, d, csc_rows, csr_ptr, deg, csr_cols);
-    CCS_CUDA_TRY(cudaGetLastError());
-    *max_deg_dev = max_deg;
+// Entries that a row (or a group of rows) with `mean` of them on average is
+// not expected to pass in a uniform draw: seven standard deviations more.
+static int likely_most(double mean, long long edges) {
+    return (int)fmin(fmin(mean + 7.0 * sqrt(mean) + 8.0, (double)edges), 2147483647.0);
+}
+
+static int bits_for(long long values) {  // of an index below `values`
+    int b = 0;
+    while (((values - 1) >> b) != 0) ++b;
+    return b;
+}
+
+static int expander_plan(int32_t n, int32_t m, int32_t d, ExpanderPlan &pl) {
+    const long long edges = (long long)n * d;
+    const double mean = (double)edges / m;
+    int dev = 0, optin = 0;
+    CCS_CUDA_TRY(cudaGetDevice(&dev));
+    CCS_CUDA_TRY(cudaDeviceGetAttribute(&pl.sms, cudaDevAttrMultiProcessorCount, dev));
+    CCS_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    pl.cap = likely_most(mean, edges);
+    if (pl.cap > kMaxSortRow) pl.cap = kMaxSortRow;
+    const int row_bits = m > 1 ? bits_for(m) : 1;
+    pl.rank_shift = ((long long)pl.cap >> (32 - row_bits)) == 0 ? row_bits : 0;
+
+    // groups of up to kGroupEntries entries, and enough of them for every SM
+    pl.groups = 0;
+    pl.col_bits = n > 1 ? bits_for(n) : 1;
+    const double target = fmin((double)kGroupEntries, fmax((double)edges / (2 * pl.sms), 1024.0));
+    int rb = 0;
+    while (rb < kMaxGroupRowBits && rb + 1 + pl.col_bits <= 32 && mean * (2 << rb) <= target &&
+           (1ll << rb) < m)
+        ++rb;
+    const long long groups = ((long long)m + (1ll << rb) - 1) >> rb;
+    pl.row_bits = rb;
+    pl.group_cap = likely_most(mean * (1 << rb), edges);
+    const double likely_row = mean + 10.0 * sqrt(mean) + 10.0;
+    if (groups > kMaxGroups || likely_row > kMaxSortRow) return CCS_OK;
+    pl.buckets = 64;
+    while (pl.buckets < pl.group_cap / 8 && pl.buckets < 8192) pl.buckets <<= 1;
+    const uint64_t span = ((uint64_t)1 << pl.col_bits) << rb;
+    pl.shift = 0;
+    while ((span >> pl.shift) > (uint64_t)pl.buckets) ++pl.shift;
+    pl.draw_smem = ((size_t)kDrawBlock * d + groups) * 4;
+    pl.sort_smem = ((size_t)pl.buckets + (1 << rb) + pl.group_cap) * 4;
+    const long long share = (edges + (long long)pl.sms * kDealBlock - 1) / ((long long)pl.sms * kDealBlock);
+    pl.deal_per = (int)(share < 1 ? 1 : (share > kDealPer ? kDealPer : share));
+    pl.deal_smem = (size_t)groups * 8 + (size_t)kDealBlock * pl.deal_per * 6;
+    if (pl.draw_smem > (size_t)optin || pl.deal_smem + 256 > (size_t)optin ||
+        pl.sort_smem + 256 > (size_t)optin)
+        return CCS_OK;
+    pl.groups = (int)groups;
     return CCS_OK;
 }
 
-// Second part: sort every CSR row ascending, given the largest row degree
-// (read back from expander_build_async).  CCS_EINVAL when a row is longer
-// than the on-chip sort takes.  Enqueued on `s`.
-int expander_sort_rows(int32_t m, int64_t *csr_ptr, int32_t *csr_cols, int host_max,
-                       cudaStream_t s) {
+// Sort every CSR row of at most `cap` columns, enqueued on `s`.  Rows of at
+// most kWarpSortCap columns: a warp a row, in registers; longer ones a block
+// a row.
+static int sort_rows(int32_t n, int32_t m, int cap, const int64_t *csr_ptr, int32_t *csr_cols,
+                     cudaStream_t s) {
+    if (cap <= kWarpSortCap) {
+        int size = 32;
+        while (size < cap) size <<= 1;
+        const int threads = 256;
+        const int grid = grid_for((long long)m * 32, threads);
+        switch (size) {
+            case 32: k_sort_rows_warp<1><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
+            case 64: k_sort_rows_warp<2><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
+            case 128: k_sort_rows_warp<4><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
+            case 256: k_sort_rows_warp<8><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
+            default: k_sort_rows_warp<16><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
+        }
+    } else {
+        int buckets = 64;
+        while (buckets < cap / 8 && buckets < 4096) buckets <<= 1;
+        int shift = 0;
+        while ((long long)(n - 1) >> shift >= buckets) ++shift;
+        const size_t smem = ((size_t)cap + buckets) * 4;
+        CCS_CUDA_TRY(cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)((kMaxSortRow + 4096) * 4)));
+        const int grid = m < 152 * 16 ? m : 152 * 16;
+        k_sort_rows<<<grid, kSortBlock, smem, s>>>(m, cap, shift, buckets, csr_ptr, csr_cols);
+    }
+    CCS_CUDA_TRY(cudaGetLastError());
+    return CCS_OK;
+}
+
+// The workspace: row degrees, block totals of their scan, the largest degree.
+struct ExpanderWs {
+    int32_t *deg;
+    int64_t *sums;
+    int *max_deg;
+    int nblocks;
+    size_t bytes;
+};
+
+static ExpanderWs expander_ws(int32_t m, void *ws) {
+    char *base = static_cast<char *>(ws);
+    ExpanderWs w;
+    w.nblocks = (int)(((long long)m + kScanBlock - 1) / kScanBlock);
+    const size_t sums = align_up((size_t)m * 4, 256);
+    const size_t top = sums + align_up((size_t)w.nblocks * 8, 256);
+    w.deg = reinterpret_cast<int32_t *>(base);
+    w.sums = reinterpret_cast<int64_t *>(base + sums);
+    w.max_deg = reinterpret_cast<int *>(base + top);
+    w.bytes = top + sizeof(int);
+    return w;
+}
+
+// The whole construction, for one d.
+template <int D>
+static int expander_build(int32_t n, int32_t m, uint64_t seed, int32_t *csc_rows,
+                          int64_t *csr_ptr, int32_t *csr_cols, const ExpanderWs &w,
+                          const ExpanderPlan &pl, cudaStream_t s) {
+    const long long edges = (long long)n * D;
+    CCS_CUDA_TRY(cudaMemsetAsync(w.deg, 0, w.bytes, s));
+    if (pl.groups) {
+        const auto big = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        CCS_CUDA_TRY(cudaFuncSetAttribute(k_draw_columns<D>, big, (int)pl.draw_smem));
+        CCS_CUDA_TRY(cudaFuncSetAttribute(k_deal_entries<D>, big, (int)pl.deal_smem));
+        CCS_CUDA_TRY(cudaFuncSetAttribute(k_sort_groups, big, (int)pl.sort_smem));
+        const int draw_grid = (int)std::min(((long long)n + kDrawBlock - 1) / kDrawBlock, 3ll * pl.sms);
+        k_draw_columns<D><<<draw_grid, kDrawBlock, pl.draw_smem, s>>>(n, m, seed, pl.row_bits,
+                                                                     pl.groups, csc_rows, w.deg);
+        k_scan_groups<<<1, kDealBlock, 0, s>>>(pl.groups, w.deg);
+        const long long turns = (edges + (long long)kDealBlock * pl.deal_per - 1) /
+                                ((long long)kDealBlock * pl.deal_per);
+        k_deal_entries<D><<<(int)std::min(turns, (long long)pl.sms), kDealBlock, pl.deal_smem, s>>>(
+            (uint32_t)edges, pl.row_bits, pl.col_bits, pl.groups, pl.deal_per, csc_rows, w.deg,
+            csr_cols);
+        k_sort_groups<<<std::min(pl.groups, 4 * pl.sms), kGroupBlock, pl.sort_smem, s>>>(
+            m, pl.groups, pl.row_bits, pl.col_bits, pl.shift, pl.buckets, pl.group_cap, w.deg,
+            csr_ptr, csr_cols, w.max_deg);
+        CCS_CUDA_TRY(cudaGetLastError());
+        return CCS_OK;
+    }
+    k_generate_columns<D><<<(n + kGenBlock - 1) / kGenBlock, kGenBlock, 0, s>>>(
+        n, m, seed, pl.rank_shift, csc_rows, w.deg);
+    k_scan_local<<<w.nblocks, kScanBlock, 0, s>>>(m, w.deg, csr_ptr, w.sums, w.max_deg);
+    k_scan_add<<<w.nblocks, kScanBlock, 0, s>>>(m, csr_ptr, w.sums);
+    CCS_CUDA_TRY(cudaGetLastError());
+    if (pl.rank_shift) {
+        k_place_ranked<D><<<grid_for((edges + 3) / 4, 256), 256, 0, s>>>(
+            edges, pl.rank_shift, csc_rows, csr_ptr, csr_cols);
+    } else {
+        CCS_CUDA_TRY(cudaMemsetAsync(w.deg, 0, (size_t)m * 4, s));
+        k_scatter_cols<<<grid_for(edges, 256), 256, 0, s>>>(n, D, csc_rows, csr_ptr, w.deg,
+                                                            csr_cols);
+    }
+    CCS_CUDA_TRY(cudaGetLastError());
+    return sort_rows(n, m, pl.cap, csr_ptr, csr_cols, s);
+}
+
+typedef int (*build_fn)(int32_t, int32_t, uint64_t, int32_t *, int64_t *, int32_t *,
+                        const ExpanderWs &, const ExpanderPlan &, cudaStream_t);
+static build_fn expander_builder(int d) {
+    static const build_fn fns[kMaxD] = {
+        expander_build<1>,  expander_build<2>,  expander_build<3>,  expander_build<4>,
+        expander_build<5>,  expander_build<6>,  expander_build<7>,  expander_build<8>,
+        expander_build<9>,  expander_build<10>, expander_build<11>, expander_build<12>,
+        expander_build<13>, expander_build<14>, expander_build<15>, expander_build<16>};
+    return fns[d - 1];
+}
+
+// The expander's whole construction, enqueued on `s` and sized for the row
+// lengths a uniform draw has.  *max_deg_dev receives the device address of
+// the largest row degree, which expander_finish needs on the host.
+// Arguments already checked.
+int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
+                         int64_t *csr_ptr, int32_t *csr_cols, void *ws, cudaStream_t s,
+                         int **max_deg_dev) {
+    ExpanderPlan pl;
+    int rc = expander_plan(n, m, d, pl);
+    if (rc) return rc;
+    const ExpanderWs w = expander_ws(m, ws);
+    *max_deg_dev = w.max_deg;
+    return expander_builder(d)(n, m, seed, csc_rows, csr_ptr, csr_cols, w, pl, s);
+}
+
+// What is left once the largest row degree is known: nothing, as a rule.
+// CCS_EINVAL when a row is longer than the on-chip sort takes.  Enqueued on
+// `s`; *again: whether anything was.
+int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
+                    int64_t *csr_ptr, int32_t *csr_cols, void *ws, int host_max, cudaStream_t s,
+                    bool *again) {
+    *again = false;
+    ExpanderPlan pl;
+    int rc = expander_plan(n, m, d, pl);
+    if (rc) return rc;
+    if (pl.groups && host_max == 0x7fffffff) {
+        // a group that did not fit on chip: build again row by row
+        const ExpanderWs w = expander_ws(m, ws);
+        pl.groups = 0;
+        if ((rc = expander_builder(d)(n, m, seed, csc_rows, csr_ptr, csr_cols, w, pl, s))) return rc;
+        CCS_CUDA_TRY(cudaMemcpyAsync(&host_max, w.max_deg, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CCS_CUDA_TRY(cudaStreamSynchronize(s));
+        *again = true;
+    }
     if (host_max > kMaxSortRow) {
         set_last_error("ccs_make_expander: a row has %d columns (limit %d)", host_max,
                        kMaxSortRow);
         return CCS_EINVAL;
     }
-    if (host_max > 1 && host_max <= 1024) {
-        // rows of at most 1024 columns: a warp a row, in registers
-        int cap = 32;
-        while (cap < host_max) cap <<= 1;
-        const int grid = 152 * 16, threads = 256;
-        switch (cap) {
-            case 32: k_sort_rows_warp<1><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-            case 64: k_sort_rows_warp<2><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-            case 128: k_sort_rows_warp<4><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-            case 256: k_sort_rows_warp<8><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-            case 512: k_sort_rows_warp<16><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-            default: k_sort_rows_warp<32><<<grid, threads, 0, s>>>(m, csr_ptr, csr_cols); break;
-        }
-        CCS_CUDA_TRY(cudaGetLastError());
-    } else if (host_max > 1) {
-        int cap = 2;
-        while (cap < host_max) cap <<= 1;
-        const size_t smem = (size_t)cap * 4;
-        if (smem > 48 * 1024)
-            CCS_CUDA_TRY(cudaFuncSetAttribute(k_sort_rows,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem));
-        const int threads = cap >= 1024 ? 1024 : (cap < 32 ? 32 : cap);
-        const int grid = m < 152 * 16 ? m : 152 * 16;
-        k_sort_rows<<<grid, threads, smem, s>>>(m, cap, csr_ptr, csr_cols);
-        CCS_CUDA_TRY(cudaGetLastError());
+    if (pl.groups || host_max <= pl.cap) return CCS_OK;
+    *again = true;
+    if (pl.rank_shift && ((long long)host_max >> (32 - pl.rank_shift)) != 0) {
+        // ranks that did not fit their bits: draw again without them
+        pl.rank_shift = 0;
+        if ((rc = expander_builder(d)(n, m, seed, csc_rows, csr_ptr, csr_cols,
+                                      expander_ws(m, ws), pl, s)))
+            return rc;
     }
-    return CCS_OK;
+    return sort_rows(n, m, host_max, csr_ptr, csr_cols, s);
 }
 
 }  // namespace ccs
@@ -551,8 +1022,10 @@ int ccs_make_expander(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *c
     int host_max = 0;
     CCS_CUDA_TRY(cudaMemcpyAsync(&host_max, max_deg, sizeof(int), cudaMemcpyDeviceToHost, s));
     CCS_CUDA_TRY(cudaStreamSynchronize(s));
-    if ((rc = expander_sort_rows(m, csr_ptr, csr_cols, host_max, s))) return rc;
-    CCS_CUDA_TRY(cudaStreamSynchronize(s));
+    bool again = false;
+    if ((rc = expander_finish(n, m, d, seed, csc_rows, csr_ptr, csr_cols, ws, host_max, s, &again)))
+        return rc;
+    if (again) CCS_CUDA_TRY(cudaStreamSynchronize(s));
     return CCS_OK;
 }
 
