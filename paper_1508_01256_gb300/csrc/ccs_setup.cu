@@ -6,6 +6,7 @@
 // is one thread's work and the matrix depends only on (n, m, d, seed).
 #include <algorithm>
 #include <cmath>
+#include <cooperative_groups.h>
 #include <cstdarg>
 #include <cstdio>
 
@@ -127,6 +128,17 @@ constexpr int kGroupEntries = 36864;  // entries a group of rows has at most, on
 constexpr int kMaxGroups = 8192;      // counted on chip
 constexpr int kMaxGroupRowBits = 12;
 constexpr int kBucketEntries = 8;
+// Matrices measured through the nonzero marks: from 2^24 entries (n = 2^22,
+// m = 2^19, d = 7: 112 us against 131 us for gathering every entry; n = 2^24,
+// m = 16777, d = 9: 193 against 604), and from 2^22 when rows are long, which
+// few warps gather (n = 2^20, m = 10486, d = 7: 25 us against 43 us).  Below,
+// x stays in L2 and the second launch costs more than it saves (n = 2^20,
+// m = 2^17, d = 7: 45 us against 37 us).
+constexpr long long kMarkedMinEntries = 1 << 24;
+constexpr long long kMarkedMinLongRows = 1 << 22;
+constexpr long long kMarkedLongRow = 128;         // mean columns of a long row
+constexpr int kMarkBytes = 128 << 10;             // marks in shared memory
+constexpr int kMarkMaxShift = 8;                  // coarsest mark: 256 columns
 
 // Per block of kScanBlock rows: inclusive prefix of deg into ptr[1 + i],
 // block total into sums[block], largest degree into *max_deg.
@@ -359,8 +371,9 @@ __global__ void k_sort_rows_warp(int m, const int64_t *ptr, int32_t *csr_cols) {
 //
 // What it replaces took two rounds of global atomics per entry, a scattered
 // 4-byte store (about 130 G/s each, whatever their size) and a sort of
-// log2(len)^2 / 2 passes: 18.2 ms at n = 2^24, m = 16777, d = 9, against
-// three passes over the entries.
+// log2(len)^2 / 2 passes: 18.2 ms at n = 2^24, m = 16777, d = 9 (2.28 ms
+// here: draw 380 us, deal 750 us, sort 1016 us) and 324 us at n = 2^20, m =
+// 2^17, d = 7 (146 us: 20, 23 and 66 us and four launches).
 
 // Columns of this block's turn, their CSC entries stored, the entries per
 // group added to size[0, groups).
@@ -499,7 +512,8 @@ k_deal_entries(uint32_t edges, int row_bits, int col_bits, int groups, int per,
 //
 // Consecutive threads hold consecutive entries, so the counting reads a
 // bucket's words together, without bank conflicts: a thread per bucket
-// sorting it by insertion took 1285 us at n = 2^24, m = 16777, d = 9.
+// sorting it by insertion took 1285 us at n = 2^24, m = 16777, d = 9, this
+// 1016 us.
 constexpr int kGroupBlock = 1024;
 __global__ void __launch_bounds__(kGroupBlock)
 k_sort_groups(int m, int groups, int row_bits, int col_bits, int shift, int buckets, int cap,
@@ -638,6 +652,142 @@ __global__ void k_measure(int m, const int64_t *ptr, const int32_t *cols, const 
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += warps) {
         const double s = warp_ordered_row_sum(ptr, cols, x, i, lane);
         if (lane == 0) y[i] = s;
+    }
+}
+
+// ---- sparse x -------------------------------------------------------------
+//
+// The signals measured are sparse (k of n entries), and a row sum skips zero
+// entries, so almost every gather of x is for nothing.  k_mark_nonzeros
+// first notes which blocks of 2^shift columns hold a nonzero (the product
+// s_j x_j for the scaled measurement), a bit each, in y's own memory;
+// k_measure_marked brings the bits into shared memory -- every CTA does,
+// before any of them stores a row of y (cooperative launch) -- and gathers
+// only where they are set.  The columns of the rows then stream at the
+// memory's rate: at n = 2^24, m = 16777, d = 9, k = 839 the 151 M gathers of
+// 32-byte sectors from 134 MB took 604 us.
+
+// A value of the measured vector: x_j, or s_j x_j rounded once.
+template <bool kScaled>
+__device__ __forceinline__ double measured_value(const double *sc, const double *x, long long j) {
+    return kScaled ? __dmul_rn(__ldg(sc + j), __ldg(x + j)) : __ldg(x + j);
+}
+
+// Bit b of `bits`: columns [b 2^shift, (b + 1) 2^shift) hold a nonzero.  A
+// warp makes whole words: 32 columns at a time, coalesced.
+template <bool kScaled>
+__global__ void k_mark_nonzeros(int n, int shift, const double *sc, const double *x,
+                                unsigned *bits) {
+    const int lane = threadIdx.x & 31;
+    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long words = (((long long)n - 1) >> shift) / 32 + 1;
+    for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < words;
+         w += warps) {
+        const long long c0 = w << (shift + 5);
+        unsigned word = 0;
+#pragma unroll 8
+        for (int u = 0; u < (1 << shift); ++u) {  // 32 columns each
+            const long long j = c0 + 32 * u + lane;
+            const bool nz = j < n && measured_value<kScaled>(sc, x, j) != 0.0;
+            const unsigned bal = __ballot_sync(0xffffffffu, nz);
+            // these 32 columns belong to 32 >> shift bits (one from shift 5 on)
+            if (shift == 0) {
+                word = bal;
+            } else if (bal) {
+                const int per = shift < 5 ? 32 >> shift : 1;
+                for (int b = 0; b < per; ++b) {
+                    const unsigned part =
+                        shift < 5 ? (bal >> (b << shift)) & ((1u << (1 << shift)) - 1u) : bal;
+                    if (part) word |= 1u << (shift < 5 ? u * per + b : u >> (shift - 5));
+                }
+            }
+        }
+        if (lane == 0) bits[w] = word;
+    }
+}
+
+// A warp takes the CTA's rows a few at a time (`batch` consecutive ones, so
+// that short rows fill its loads too) and streams their columns; set bits
+// are looked up in order, so a row's nonzero values are added in ascending
+// j from +0.0, as in warp_ordered_row_sum.
+constexpr int kMarkBlock = 1024;
+constexpr int kMarkUnroll = 8;  // (12 and 16: 2 and 13 % slower)
+template <bool kScaled>
+__global__ void __launch_bounds__(kMarkBlock)
+k_measure_marked(int m, int shift, int words, int batch, const int64_t *ptr, const int32_t *cols,
+                 const double *sc, const double *x, double *y) {
+    extern __shared__ unsigned bits[];
+    __shared__ int next;
+    const unsigned *src = reinterpret_cast<const unsigned *>(y);
+    for (int w = threadIdx.x; w < words; w += kMarkBlock) bits[w] = __ldcg(src + w);
+    const int lane = threadIdx.x & 31;
+    const int r0 = (int)((long long)m * blockIdx.x / gridDim.x);
+    const int r1 = (int)((long long)m * (blockIdx.x + 1) / gridDim.x);
+    if (threadIdx.x == 0) next = r0;
+    cooperative_groups::this_grid().sync();
+    for (;;) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(&next, batch);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= r1) break;
+        const int rows = min(batch, r1 - i);  // at most 32: lane l keeps the end of row i + l
+        const int64_t b = __ldg(ptr + i);
+        const int64_t mine = __ldg(ptr + i + 1 + min(lane, rows - 1));
+        const int64_t e = __shfl_sync(0xffffffffu, mine, rows - 1);
+        int row = 0;
+        int64_t row_end = __shfl_sync(0xffffffffu, mine, 0);
+        double s = 0.0, out = 0.0;  // lane l: the finished sum of row i + l
+        int c[kMarkUnroll];
+#pragma unroll
+        for (int u = 0; u < kMarkUnroll; ++u) {
+            const int64_t p = b + 32 * u + lane;
+            c[u] = p < e ? __ldcs(cols + p) : -1;
+        }
+        for (int64_t p0 = b; p0 < e; p0 += 32 * kMarkUnroll) {
+            int cn[kMarkUnroll];
+#pragma unroll
+            for (int u = 0; u < kMarkUnroll; ++u) {
+                const int64_t p = p0 + 32 * (kMarkUnroll + u) + lane;
+                cn[u] = p < e ? __ldcs(cols + p) : -1;
+            }
+            unsigned hit = 0;
+#pragma unroll
+            for (int u = 0; u < kMarkUnroll; ++u) {
+                const unsigned blk = (unsigned)max(c[u], 0) >> shift;
+                hit |= (c[u] >= 0 ? (bits[blk >> 5] >> (blk & 31)) & 1u : 0u) << u;
+            }
+            if (__any_sync(0xffffffffu, hit)) {
+                constexpr int kV = 4;  // gathers in flight
+#pragma unroll
+                for (int u0 = 0; u0 < kMarkUnroll; u0 += kV) {
+                    double v[kV];
+#pragma unroll
+                    for (int u = 0; u < kV; ++u)
+                        v[u] = (hit >> (u0 + u)) & 1u ? measured_value<kScaled>(sc, x, c[u0 + u])
+                                                      : 0.0;
+#pragma unroll
+                    for (int u = 0; u < kV; ++u) {
+                        unsigned nz = __ballot_sync(0xffffffffu, v[u] != 0.0);
+                        while (nz) {
+                            const int at = __ffs(nz) - 1;
+                            nz &= nz - 1;
+                            const int64_t p = p0 + 32 * (u0 + u) + at;
+                            while (p >= row_end) {  // rows that end before this entry
+                                if (lane == row) out = s;
+                                s = 0.0;
+                                ++row;
+                                row_end = __shfl_sync(0xffffffffu, mine, row);
+                            }
+                            s = __dadd_rn(s, __shfl_sync(0xffffffffu, v[u], at));
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kMarkUnroll; ++u) c[u] = cn[u];
+        }
+        if (lane == row) out = s;  // later rows hold no nonzero: 0.0
+        if (lane < rows) y[i + lane] = out;
     }
 }
 
@@ -981,6 +1131,49 @@ int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc
     return sort_rows(n, m, host_max, csr_ptr, csr_cols, s);
 }
 
+// y = A x or y = A diag(sc) x, enqueued on `s`: through the nonzero marks
+// when the matrix is large, else by gathering every entry.
+template <bool kScaled>
+static int measure_rows(int32_t n, int32_t m, int32_t d, const int64_t *csr_ptr,
+                        const int32_t *csr_cols, const double *sc, const double *x, double *y,
+                        cudaStream_t s) {
+    const long long edges = (long long)n * d;
+    if (edges >= kMarkedMinEntries ||
+        (edges >= kMarkedMinLongRows && edges / m >= kMarkedLongRow)) {
+        int dev = 0, sms = 0, coop = 0;
+        CCS_CUDA_TRY(cudaGetDevice(&dev));
+        CCS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        CCS_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        // as many bits as y (64 m) and shared memory hold
+        const long long room = std::min(64ll * m, (long long)kMarkBytes * 8);
+        int shift = 0;
+        while (((((long long)n - 1) >> shift) / 32 + 1) * 32 > room) ++shift;
+        const int words = (int)((((long long)n - 1) >> shift) / 32 + 1);
+        if (coop && shift <= kMarkMaxShift) {
+            k_mark_nonzeros<kScaled><<<sms * 8, 256, 0, s>>>(n, shift, sc, x,
+                                                             reinterpret_cast<unsigned *>(y));
+            CCS_CUDA_TRY(cudaGetLastError());
+            const size_t smem = (size_t)words * 4;
+            CCS_CUDA_TRY(cudaFuncSetAttribute(k_measure_marked<kScaled>,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              kMarkBytes));
+            int batch = (int)std::max(1ll, std::min(32ll, 512ll * m / edges));
+            int words_arg = words, shift_arg = shift;
+            void *args[] = {&m, &shift_arg, &words_arg, &batch, &csr_ptr, &csr_cols, &sc, &x, &y};
+            CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)k_measure_marked<kScaled>,
+                                                     dim3(sms), dim3(kMarkBlock), args, smem, s));
+            return CCS_OK;
+        }
+    }
+    const long long threads = (long long)m * 32;
+    if (kScaled)
+        k_measure_scaled<<<grid_for(threads, 256), 256, 0, s>>>(m, csr_ptr, csr_cols, sc, x, y);
+    else
+        k_measure<<<grid_for(threads, 256), 256, 0, s>>>(m, csr_ptr, csr_cols, x, y);
+    CCS_CUDA_TRY(cudaGetLastError());
+    return CCS_OK;
+}
+
 }  // namespace ccs
 
 extern "C" {
@@ -1030,10 +1223,7 @@ int ccs_measure(int32_t n, int32_t m, int32_t d, const int64_t *csr_ptr,
         (rc = check_aligned("ccs_measure", "x", x, 8)))
         return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const long long threads = (long long)m * 32;
-    k_measure<<<grid_for(threads, 256), 256, 0, s>>>(m, csr_ptr, csr_cols, x, y);
-    CCS_CUDA_TRY(cudaGetLastError());
-    return CCS_OK;
+    return measure_rows<false>(n, m, d, csr_ptr, csr_cols, nullptr, x, y, s);
 }
 
 int ccs_column_scales(int32_t n, uint64_t seed, double *scales, ccs_stream_t stream) {
@@ -1063,10 +1253,7 @@ int ccs_measure_scaled(int32_t n, int32_t m, int32_t d, const int64_t *csr_ptr,
         (rc = check_aligned("ccs_measure_scaled", "s", scales, 8)))
         return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const long long threads = (long long)m * 32;
-    k_measure_scaled<<<grid_for(threads, 256), 256, 0, s>>>(m, csr_ptr, csr_cols, scales, x, y);
-    CCS_CUDA_TRY(cudaGetLastError());
-    return CCS_OK;
+    return measure_rows<true>(n, m, d, csr_ptr, csr_cols, scales, x, y, s);
 }
 
 int ccs_unscale(int32_t n, const double *scales, const double *z, double *x,
