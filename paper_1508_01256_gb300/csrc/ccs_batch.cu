@@ -8,6 +8,9 @@
 
 namespace ccs {
 
+// Most problems of a batch: a launch of the persistent engine takes no more.
+constexpr int kMaxBatch = 4096;
+
 // Iterations each launch group of a batch runs alone before the launch that
 // merges the groups' tails (most converging problems finish within it).
 constexpr int kGroupIters = 16;
@@ -136,6 +139,10 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
                                        pr.r, pr.r0_hist)))
             return rc;
     }
+    if (count > kMaxBatch) {
+        set_last_error("at most %d problems per launch (got %d)", kMaxBatch, count);
+        return CCS_EINVAL;
+    }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     char *hdr = static_cast<char *>(ws);
     char *rhdr = hdr + engine_header_bytes(count);
@@ -175,56 +182,50 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
         }
         return CCS_OK;
     }
-    // A batch goes out as up to four launches, one per class, each over the
-    // whole GPU: d <= 8 and d > 8 run on different kernel instances (the
-    // register-resident arrays are sized by the largest d of a launch), and
-    // problems whose fingerprints do not fit shared memory would shrink every
-    // other problem's launch plan (fewer stages, a smaller queue) and its
-    // thread count.  Every problem's result is the same either way.
+    // Problems that fit a cluster on chip go out in one launch of the small
+    // engine.  The others go out as up to four launches, one per class, each
+    // over the whole GPU: d <= 8 and d > 8 run on different kernel instances
+    // (the register-resident arrays are sized by the largest d of a launch),
+    // and problems whose fingerprints do not fit shared memory would shrink
+    // every other problem's launch plan (fewer stages, a smaller queue) and
+    // its thread count.  Every problem's result is the same either way.
+    constexpr int kSmallClass = 4;
     std::vector<int> cls(count);
     for (int32_t q = 0; q < count; ++q)
-        cls[q] = (pds[q].d > 8 ? 2 : 0) + (engine_fp_fits(pds[q], p) ? 0 : 1);
-    std::vector<int> order;
+        cls[q] = !tuned && small_route(pds[q], p, count == 1)
+                     ? kSmallClass
+                     : (pds[q].d > 8 ? 2 : 0) + (engine_fp_fits(pds[q], p) ? 0 : 1);
+    // descriptors in launch order; out_slot keeps the caller's index
+    std::vector<ProblemDev> sub;
     int sizes[4] = {0, 0, 0, 0};
     int groups = 0;
-    for (int c = 0; c < 4; ++c) {
-        int cnt = 0;
+    for (int c = 0; c <= kSmallClass; ++c) {
+        const size_t before = sub.size();
         for (int32_t q = 0; q < count; ++q)
             if (cls[q] == c) {
-                order.push_back(q);
-                ++cnt;
+                sub.push_back(pds[q]);
+                sub.back().ctrl = header_ctrl(hdr, (int)sub.size() - 1);
             }
-        if (cnt) sizes[groups++] = cnt;
+        if (c < kSmallClass && sub.size() > before) sizes[groups++] = (int)(sub.size() - before);
     }
-    // descriptors in launch order; each launch's control blocks sit at the
-    // front of the header, and out_slot keeps the caller's index
-    std::vector<ProblemDev> sub(count);
-    for (int g = 0, t = 0; g < groups; ++g)
-        for (int u = 0; u < sizes[g]; ++u, ++t) {
-            sub[t] = pds[order[t]];
-            sub[t].ctrl = header_ctrl(hdr, u);
-        }
-    std::vector<ccs_result> part(count);
-    if (tuned) return autotune_groups(sub, sizes, groups, p, hdr, s, tuned);
-    if (groups > 1) {
-        // each group alone for its first iterations, then one launch over the
-        // whole batch for the problems still running, so that the groups'
-        // tails (problems that iterate to max_iter) overlap
-        for (int t = 0; t < count; ++t) sub[t].ctrl = header_ctrl(hdr, t);
-        if (capture)
-            return engine_capture_phased(sub.data(), sizes, groups, count, p, kGroupIters, hdr,
-                                         rhdr, dev_out, capture);
-        return engine_run_phased(sub.data(), sizes, groups, count, p, kGroupIters, hdr, rhdr, s,
-                                 dev_out, out);
+    // the small engine's clusters take the largest problems first
+    int rest = 0;
+    for (int g = 0; g < groups; ++g) rest += sizes[g];
+    std::stable_sort(sub.begin() + rest, sub.end(), [](const ProblemDev &x, const ProblemDev &y) {
+        return (long long)x.n * x.d > (long long)y.n * y.d;
+    });
+    if (tuned) {
+        // each launch's control blocks sit at the front of the header
+        for (int g = 0, t = 0; g < groups; ++g)
+            for (int u = 0; u < sizes[g]; ++u, ++t) sub[t].ctrl = header_ctrl(hdr, u);
+        return autotune_groups(sub, sizes, groups, p, hdr, s, tuned);
     }
-    if (capture) return engine_capture(sub.data(), sizes, groups, p, hdr, dev_out, capture);
-    for (int g = 0, first = 0; g < groups; first += sizes[g], ++g) {
-        rc = engine_run(sub.data() + first, sizes[g], p, part.data() + first, hdr, s, dev_out);
-        if (rc != CCS_OK) return rc;
-    }
-    if (!dev_out)
-        for (int t = 0; t < count; ++t) out[order[t]] = part[t];
-    return CCS_OK;
+    ccs_result *res =
+        dev_out ? dev_out : reinterpret_cast<ccs_result *>(rhdr + sizeof(EngineSync));
+    if ((rc = engine_run_batch(sub.data(), sizes, groups, count, p, kGroupIters, hdr, rhdr, s, res,
+                               capture)))
+        return rc;
+    return dev_out ? CCS_OK : engine_results(rhdr, count, out, s);
 }
 
 extern "C" int ccs_decode_batch(const ccs_problem *probs, int32_t count, const ccs_params *params,

@@ -317,8 +317,9 @@ bool engine_fp_fits(const ProblemDev &pd, const ccs_params &prm) {
 
 int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, char *ws,
                cudaStream_t s, ccs_result *dev_out) {
-    LaunchPlan L;
-    int rc = plan_launch(pds, P, prm, L);
+    const bool small = P == 1 && small_route(pds[0], prm, true);
+    LaunchPlan L{};
+    int rc = small ? CCS_OK : plan_launch(pds, P, prm, L);
     if (rc) return rc;
     EngineArgs a;
     fill_args(a, L, P, prm);
@@ -326,7 +327,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     char *e = ws + sync_bytes(P);
     unsigned long long *stamps = reinterpret_cast<unsigned long long *>(e);
     e += stamps_bytes();
-    a.stamps = (profiling() && !dev_out) ? stamps : nullptr;
+    a.stamps = (profiling() && !dev_out && !small) ? stamps : nullptr;
     a.dev_out = dev_out;
     if (a.stamps) CCS_CUDA_TRY(cudaMemsetAsync(stamps, 0, stamps_bytes(), s));
 
@@ -344,12 +345,18 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
         a.probs = d_probs;
     }
 
-    void *args[] = {&a};
-    const int ev = prof_start(CCS_K_PERSISTENT, s);
-    CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads), args,
-                                             L.smem, s));
-    prof_stop(ev, s);
-    count_launches(1);
+    if (small) {
+        if ((rc = small_launch(pds, nullptr, 1, prm, false, 0x7fffffff, a.sync, dev_out, s,
+                               true)))
+            return rc;
+    } else {
+        void *args[] = {&a};
+        const int ev = prof_start(CCS_K_PERSISTENT, s);
+        CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
+                                                 args, L.smem, s));
+        prof_stop(ev, s);
+        count_launches(1);
+    }
     if (dev_out) return CCS_OK;  // asynchronous: the kernel writes the results
 
     // results: one copy of the sync word and every control block (a stack
@@ -415,62 +422,6 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     return CCS_OK;
 }
 
-// Capture decode launches (header memset + cooperative kernel, one pair per
-// group, run one after the other) into a CUDA graph.  pds holds the groups'
-// descriptors back to back, group g's sizes[g] of them, each with its control
-// block at the group's own index in the header.  The descriptors are uploaded
-// now, outside the capture, to disjoint places of the header; the graph bakes
-// the workspace and array pointers.  Results go to dev_out.
-int engine_capture(ProblemDev *pds, const int *sizes, int groups, const ccs_params &prm, char *ws,
-                   ccs_result *dev_out, cudaGraphExec_t *exec) {
-    int total = 0;
-    for (int g = 0; g < groups; ++g) total += sizes[g];
-    std::vector<EngineArgs> args(groups);
-    std::vector<LaunchPlan> plans(groups);
-    ProblemDev *d_probs = reinterpret_cast<ProblemDev *>(ws + sync_bytes(total) + stamps_bytes());
-    for (int g = 0, first = 0; g < groups; first += sizes[g], ++g) {
-        const int P = sizes[g];
-        int rc = plan_launch(pds + first, P, prm, plans[g]);
-        if (rc) return rc;
-        EngineArgs &a = args[g];
-        fill_args(a, plans[g], P, prm);
-        a.sync = reinterpret_cast<EngineSync *>(ws);
-        a.dev_out = dev_out;
-        a.stamps = nullptr;
-        if (P == 1) {
-            a.single = pds[first];
-            a.probs = nullptr;
-        } else {
-            a.probs = d_probs + first;
-        }
-    }
-    // upload the descriptors with the flags plan_launch set
-    if (total > 1)
-        CCS_CUDA_TRY(cudaMemcpy(d_probs, pds, sizeof(ProblemDev) * total, cudaMemcpyHostToDevice));
-    cudaStream_t cs;
-    CCS_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        cudaError_t e1 = cudaSuccess;
-        for (int g = 0; g < groups && e1 == cudaSuccess; ++g) {
-            const LaunchPlan &L = plans[g];
-            void *kargs[] = {&args[g]};
-            e1 = cudaMemsetAsync(ws, 0, sync_bytes(sizes[g]), cs);
-            if (e1 == cudaSuccess)
-                e1 = cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
-                                                 kargs, L.smem, cs);
-        }
-        e = cudaStreamEndCapture(cs, &graph);
-        if (e == cudaSuccess) e = e1;
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    cudaStreamDestroy(cs);
-    if (e != cudaSuccess) return cuda_fail(e, "capturing the engine launch");
-    return CCS_OK;
-}
-
 // Resume-mode header: [EngineSync | P ccs_result] [stamps] [P descriptors].
 static size_t resume_results_bytes(int P) {
     return align_up(sizeof(EngineSync) + sizeof(ccs_result) * (size_t)P, 256);
@@ -480,139 +431,115 @@ size_t engine_resume_header_bytes(int P) {
     return resume_results_bytes(P) + stamps_bytes() + align_up(sizeof(ProblemDev) * (size_t)P, 256);
 }
 
-// Enqueue one resume-mode launch (no host wait).  Results go to dev_out,
-// each at its problem's out_slot, or to the header's result area.
-static int engine_resume_launch(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget,
-                                char *hdr, cudaStream_t s, ccs_result *dev_out) {
-    LaunchPlan L;
-    int rc = plan_launch(pds, P, prm, L);
-    if (rc) return rc;
-    EngineArgs a;
-    fill_args(a, L, P, prm);
-    a.resume = 1;
-    a.iter_budget = iter_budget > 0 ? iter_budget : 1;
-    a.sync = reinterpret_cast<EngineSync *>(hdr);
-    a.dev_out = dev_out ? dev_out : reinterpret_cast<ccs_result *>(hdr + sizeof(EngineSync));
-    ProblemDev *d_probs =
-        reinterpret_cast<ProblemDev *>(hdr + resume_results_bytes(P) + stamps_bytes());
-    a.probs = d_probs;
-    CCS_CUDA_TRY(cudaMemsetAsync(hdr, 0, sizeof(EngineSync), s));
-    CCS_CUDA_TRY(cudaMemcpyAsync(d_probs, pds, sizeof(ProblemDev) * P, cudaMemcpyHostToDevice, s));
-    void *args[] = {&a};
-    const int ev = prof_start(CCS_K_PERSISTENT, s);
-    CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads), args,
-                                             L.smem, s));
-    prof_stop(ev, s);
-    count_launches(1);
-    return CCS_OK;
-}
-
-// A batch whose launch classes (groups) would each end in their own long
-// tail of problems that iterate to max_iter: every group first runs alone,
+// A batch.  pds: the `rest` = sum of sizes[0..groups) problems of the launch
+// classes back to back, then the count - rest that go out as one launch of
+// the small engine; their out_slot the caller's index, their control blocks
+// distinct, in `hdr` (engine_header_bytes(count)); rhdr:
+// engine_resume_header_bytes(count) bytes.
+//
+// Launch classes (groups) would each end in their own long tail of problems
+// that iterate to max_iter: with several, every group first runs alone,
 // freshly initialised, for at most group_iters iterations; then one launch
-// over every problem of the batch resumes the ones still running, so the
-// groups' tails share iterations.  pds: the groups' descriptors back to back
-// (their out_slot the caller's index, their control blocks distinct, in
-// `ctrl_hdr`, `count` of them); rhdr: engine_resume_header_bytes(count)
-// bytes.  Results: dev_out (each at out_slot), or host_out[out_slot].
-int engine_run_phased(ProblemDev *pds, const int *sizes, int groups, int count,
-                      const ccs_params &prm, int group_iters, char *ctrl_hdr, char *rhdr,
-                      cudaStream_t s, ccs_result *dev_out, ccs_result *host_out) {
-    CCS_CUDA_TRY(cudaMemsetAsync(ctrl_hdr, 0, sync_bytes(count), s));
-    for (int t = 0; t < count; ++t) pds[t].flags |= kPdFresh;
-    for (int g = 0, first = 0; g < groups; first += sizes[g], ++g) {
-        int rc = engine_resume_launch(pds + first, sizes[g], prm, group_iters, rhdr, s, nullptr);
-        if (rc) return rc;
-    }
-    for (int t = 0; t < count; ++t) pds[t].flags &= ~kPdFresh;
-    int rc = engine_resume_launch(pds, count, prm, 0x7fffffff, rhdr, s, dev_out);
-    if (rc || dev_out) return rc;
-    const size_t bytes = sizeof(EngineSync) + sizeof(ccs_result) * (size_t)count;
-    std::vector<char> h(bytes);
-    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), rhdr, bytes, cudaMemcpyDeviceToHost, s));
-    CCS_CUDA_TRY(cudaStreamSynchronize(s));
-    EngineSync hs;
-    std::memcpy(&hs, h.data(), sizeof(hs));
-    std::memcpy(host_out, h.data() + sizeof(EngineSync), sizeof(ccs_result) * (size_t)count);
-    if (hs.error) {
-        for (int t = 0; t < count; ++t) host_out[t].error = CCS_ETIMEOUT;
-        set_last_error("a bounded device wait exceeded the watchdog");
-        return CCS_ETIMEOUT;
-    }
-    return CCS_OK;
-}
-
-// engine_run_phased captured in a CUDA graph: the control blocks' reset,
-// each group's capped launch and the final launch over the whole batch.
-// The descriptors are uploaded now, outside the capture: the groups' (fresh)
-// to the launch header's descriptor area, the final launch's to the resume
-// header's.  Results of the final launch go to dev_out.
-int engine_capture_phased(ProblemDev *pds, const int *sizes, int groups, int count,
-                          const ccs_params &prm, int group_iters, char *ctrl_hdr, char *rhdr,
-                          ccs_result *dev_out, cudaGraphExec_t *exec) {
-    std::vector<ProblemDev> fresh(pds, pds + count), resumed(pds, pds + count);
+// over all of them resumes the ones still running, so the tails share
+// iterations.
+//
+// Results go to res[out_slot].  Enqueued on `s`, or, with `capture`, made a
+// CUDA graph that replays the launches (the descriptors are uploaded now).
+int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
+                     const ccs_params &prm, int group_iters, char *hdr, char *rhdr,
+                     cudaStream_t s, ccs_result *res, cudaGraphExec_t *capture) {
+    int rest = 0;
+    for (int g = 0; g < groups; ++g) rest += sizes[g];
+    ProblemDev *d_fresh = reinterpret_cast<ProblemDev *>(hdr + sync_bytes(count) + stamps_bytes());
+    ProblemDev *d_again =
+        reinterpret_cast<ProblemDev *>(rhdr + resume_results_bytes(count) + stamps_bytes());
+    EngineSync *sync = reinterpret_cast<EngineSync *>(rhdr);
+    const int launches = groups > 1 ? groups + 1 : groups;
+    std::vector<ProblemDev> fresh(pds, pds + count), again(pds, pds + count);
     for (int t = 0; t < count; ++t) {
         fresh[t].flags |= kPdFresh;
-        resumed[t].flags &= ~kPdFresh;
+        again[t].flags &= ~kPdFresh;
     }
-    ProblemDev *d_fresh =
-        reinterpret_cast<ProblemDev *>(ctrl_hdr + sync_bytes(count) + stamps_bytes());
-    ProblemDev *d_resumed =
-        reinterpret_cast<ProblemDev *>(rhdr + resume_results_bytes(count) + stamps_bytes());
-    std::vector<EngineArgs> args(groups + 1);
-    std::vector<LaunchPlan> plans(groups + 1);
-    for (int g = 0, first = 0; g <= groups; ++g) {
-        const bool last = g == groups;
-        const int P = last ? count : sizes[g];
-        ProblemDev *host = last ? resumed.data() : fresh.data() + first;
-        int rc = plan_launch(host, P, prm, plans[g]);
+    std::vector<EngineArgs> args(launches);
+    std::vector<LaunchPlan> plans(launches);
+    for (int l = 0, first = 0; l < launches; ++l) {
+        const bool last = l == launches - 1, tail = l == groups;
+        const int P = tail ? rest : sizes[l];
+        ProblemDev *host = tail ? again.data() : fresh.data() + first;
+        int rc = plan_launch(host, P, prm, plans[l]);
         if (rc) return rc;
-        EngineArgs &a = args[g];
-        fill_args(a, plans[g], P, prm);
-        a.resume = 1;
-        a.iter_budget = last ? 0x7fffffff : (group_iters > 0 ? group_iters : 1);
-        a.sync = reinterpret_cast<EngineSync *>(rhdr);
-        a.dev_out = last ? dev_out : reinterpret_cast<ccs_result *>(rhdr + sizeof(EngineSync));
-        a.stamps = nullptr;
-        a.probs = last ? d_resumed : d_fresh + first;
-        if (!last) first += sizes[g];
+        EngineArgs &a = args[l];
+        fill_args(a, plans[l], P, prm);
+        a.sync = sync;
+        a.dev_out = last ? res : nullptr;
+        if (rest == 1) {
+            a.single = *host;  // a lone problem
+        } else {
+            a.resume = 1;
+            a.iter_budget = last ? 0x7fffffff : (group_iters > 0 ? group_iters : 1);
+            a.probs = tail ? d_again : d_fresh + first;
+        }
+        if (!tail) first += sizes[l];
     }
-    // upload with the flags plan_launch set
-    CCS_CUDA_TRY(cudaMemcpy(d_fresh, fresh.data(), sizeof(ProblemDev) * count,
-                            cudaMemcpyHostToDevice));
-    CCS_CUDA_TRY(cudaMemcpy(d_resumed, resumed.data(), sizeof(ProblemDev) * count,
-                            cudaMemcpyHostToDevice));
+    // upload with the flags plan_launch set (count == 1: a single problem
+    // travels with its launch, and the header has no room for descriptors)
+    if (count > 1) {
+        const size_t bytes = sizeof(ProblemDev) * (size_t)count;
+        if (capture) {
+            CCS_CUDA_TRY(cudaMemcpy(d_fresh, fresh.data(), bytes, cudaMemcpyHostToDevice));
+            CCS_CUDA_TRY(cudaMemcpy(d_again, again.data(), bytes, cudaMemcpyHostToDevice));
+        } else {
+            CCS_CUDA_TRY(cudaMemcpyAsync(d_fresh, fresh.data(), bytes, cudaMemcpyHostToDevice, s));
+            if (groups > 1)
+                CCS_CUDA_TRY(cudaMemcpyAsync(d_again, again.data(), bytes, cudaMemcpyHostToDevice, s));
+        }
+    }
+    auto enqueue = [&](cudaStream_t cs) -> int {
+        CCS_CUDA_TRY(cudaMemsetAsync(hdr, 0, sync_bytes(count), cs));
+        CCS_CUDA_TRY(cudaMemsetAsync(sync, 0, sizeof(EngineSync), cs));
+        int rc;
+        if (rest < count &&
+            (rc = small_launch(pds + rest, count > 1 ? d_fresh + rest : nullptr, count - rest, prm,
+                               false, 0x7fffffff, sync, res, cs, !capture)))
+            return rc;
+        for (int l = 0; l < launches; ++l) {
+            const LaunchPlan &L = plans[l];
+            // the barrier starts at zero; a launch keeps the error bits of the ones before
+            if (l) CCS_CUDA_TRY(cudaMemsetAsync(&sync->arrive, 0, sizeof(sync->arrive), cs));
+            void *kargs[] = {&args[l]};
+            const int ev = capture ? -1 : prof_start(CCS_K_PERSISTENT, cs);
+            CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
+                                                     kargs, L.smem, cs));
+            if (!capture) {
+                prof_stop(ev, cs);
+                count_launches(1);
+            }
+        }
+        return CCS_OK;
+    };
+    if (!capture) return enqueue(s);
     cudaStream_t cs;
     CCS_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
+    int rc = CCS_OK;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e1 = cudaMemsetAsync(ctrl_hdr, 0, sync_bytes(count), cs);
-        for (int g = 0; g <= groups && e1 == cudaSuccess; ++g) {
-            const LaunchPlan &L = plans[g];
-            void *kargs[] = {&args[g]};
-            e1 = cudaMemsetAsync(rhdr, 0, sizeof(EngineSync), cs);
-            if (e1 == cudaSuccess)
-                e1 = cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
-                                                 kargs, L.smem, cs);
-        }
+        rc = enqueue(cs);
         e = cudaStreamEndCapture(cs, &graph);
-        if (e == cudaSuccess) e = e1;
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(exec, graph, 0);
+    if (e == cudaSuccess && rc == CCS_OK) e = cudaGraphInstantiate(capture, graph, 0);
     if (graph) cudaGraphDestroy(graph);
     cudaStreamDestroy(cs);
-    if (e != cudaSuccess) return cuda_fail(e, "capturing the phased batch");
+    if (rc) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, "capturing the batch");
     return CCS_OK;
 }
 
-int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
-                  char *hdr, cudaStream_t s) {
-    int rc = engine_resume_launch(pds, P, prm, iter_budget, hdr, s, nullptr);
-    if (rc) return rc;
+// The result area of a header (P entries) to the host.  Waits for `s`.
+int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s) {
     const size_t bytes = sizeof(EngineSync) + sizeof(ccs_result) * (size_t)P;
     std::vector<char> h(bytes);
-    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), hdr, bytes, cudaMemcpyDeviceToHost, s));
+    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), rhdr, bytes, cudaMemcpyDeviceToHost, s));
     CCS_CUDA_TRY(cudaStreamSynchronize(s));
     EngineSync hs;
     std::memcpy(&hs, h.data(), sizeof(hs));
@@ -623,6 +550,43 @@ int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget
         return CCS_ETIMEOUT;
     }
     return CCS_OK;
+}
+
+// A server round.  Problems that fit a cluster on chip go out in a launch of
+// their own.  pds: out_slot 0..P-1, in any order.
+int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
+                  char *hdr, cudaStream_t s) {
+    const int rest = (int)(std::stable_partition(pds, pds + P, [&](const ProblemDev &q) {
+                               return !small_route(q, prm, P == 1);
+                           }) - pds);
+    EngineSync *sync = reinterpret_cast<EngineSync *>(hdr);
+    ccs_result *res = reinterpret_cast<ccs_result *>(hdr + sizeof(EngineSync));
+    ProblemDev *d_probs =
+        reinterpret_cast<ProblemDev *>(hdr + resume_results_bytes(P) + stamps_bytes());
+    LaunchPlan L{};
+    int rc;
+    if (rest && (rc = plan_launch(pds, rest, prm, L))) return rc;
+    CCS_CUDA_TRY(cudaMemsetAsync(sync, 0, sizeof(EngineSync), s));
+    CCS_CUDA_TRY(cudaMemcpyAsync(d_probs, pds, sizeof(ProblemDev) * P, cudaMemcpyHostToDevice, s));
+    if (rest < P && (rc = small_launch(pds + rest, d_probs + rest, P - rest, prm, true,
+                                       iter_budget, sync, res, s, true)))
+        return rc;
+    if (rest) {
+        EngineArgs a;
+        fill_args(a, L, rest, prm);
+        a.resume = 1;
+        a.iter_budget = iter_budget > 0 ? iter_budget : 1;
+        a.sync = sync;
+        a.dev_out = res;
+        a.probs = d_probs;
+        void *args[] = {&a};
+        const int ev = prof_start(CCS_K_PERSISTENT, s);
+        CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
+                                                 args, L.smem, s));
+        prof_stop(ev, s);
+        count_launches(1);
+    }
+    return engine_results(hdr, P, out, s);
 }
 
 }  // namespace ccs

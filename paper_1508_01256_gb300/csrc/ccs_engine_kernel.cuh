@@ -51,8 +51,6 @@ constexpr int kOvfCap = 512;       // overflow rows listed per CTA and segment
 constexpr int kQueueCap = 2048;     // most candidate columns queued per CTA and segment
 constexpr int kMinQueue = 256;      // fewest (more go through the inline exact path)
 constexpr int kFlagSkipArrive = 1;  // test hook: CTA 0 never arrives at barrier 1
-constexpr int kFlagOrdered = 2;     // test hook: ordered residual from the start
-constexpr int kFlagSwitch = 4;      // test hook: the certificate fails from iteration 2
 constexpr int kFlagRowInline = 8;   // test hook: row-driven candidates scored inline, no queue
 constexpr int kFlagRowAlways = 16;  // test hook: row-driven whenever the row list fits
 constexpr int kFlagRowNever = 32;   // every score phase streams the CSC

@@ -16,6 +16,11 @@ constexpr int kSlotRec = 16;        // ints per row record: count, then kSlots c
 constexpr int kMaxSortRow = 32768;  // longest CSR row sorted on chip
 constexpr int kRunning = -1;        // DecodeCtrl::status while iterating
 
+// Bits of ccs_params.debug_flags that both engines know (the others are in
+// ccs_engine_kernel.cuh).
+constexpr int kFlagOrdered = 2;     // test hook: ordered residual from the start
+constexpr int kFlagSwitch = 4;      // test hook: the certificate fails from iteration 2
+
 enum ProblemFlags : int {
     kPdUseFp = 1,
     kPdFresh = 2,
@@ -124,7 +129,8 @@ __host__ inline size_t decode_ws_layout(int n, int m, ProblemDev *pd, char *base
 struct alignas(64) EngineSync {
     unsigned arrive;  // monotonic grid-barrier counter
     int error;        // ErrorBits of the launch
-    int pad[14];
+    unsigned next;    // problems taken by the small engine's clusters
+    int pad[13];
 };
 static_assert(sizeof(EngineSync) == 64, "EngineSync layout");
 
@@ -197,10 +203,14 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
 // iter_budget iterations run; out[p].status is -1 for problems still
 // running.  `hdr` needs engine_resume_header_bytes(P) bytes.
 size_t engine_resume_header_bytes(int P);
-// Graph of `groups` launches run in turn; pds holds group g's sizes[g]
-// descriptors after those of the groups before it.
-int engine_capture(ProblemDev *pds, const int *sizes, int groups, const ccs_params &prm, char *ws,
-                   ccs_result *dev_out, cudaGraphExec_t *exec);
+// Small problems (ccs_small.cu): decoded by one thread-block cluster each, on
+// chip.  small_route: whether a problem takes that path under these params
+// (alone: nothing else shares the GPU with it).
+bool small_route(const ProblemDev &pd, const ccs_params &prm, bool alone);
+int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_params &prm,
+                 bool resume, int iter_budget, EngineSync *sync, ccs_result *dev_out,
+                 cudaStream_t s, bool timed);
+
 // The expander's construction (ccs_setup.cu): all of it enqueued, then what
 // the largest row degree, read back by the caller, may still ask for.
 int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
@@ -212,14 +222,12 @@ int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc
 
 int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
                   char *hdr, cudaStream_t s);
-// A multi-group batch with merged tails (see ccs_engine.cu), run now or
-// captured in a CUDA graph.
-int engine_run_phased(ProblemDev *pds, const int *sizes, int groups, int count,
-                      const ccs_params &prm, int group_iters, char *ctrl_hdr, char *rhdr,
-                      cudaStream_t s, ccs_result *dev_out, ccs_result *host_out);
-int engine_capture_phased(ProblemDev *pds, const int *sizes, int groups, int count,
-                          const ccs_params &prm, int group_iters, char *ctrl_hdr, char *rhdr,
-                          ccs_result *dev_out, cudaGraphExec_t *exec);
+// A batch (see ccs_engine.cu), run now or captured in a CUDA graph, and the
+// read-back of a header's results.
+int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
+                     const ccs_params &prm, int group_iters, char *hdr, char *rhdr,
+                     cudaStream_t s, ccs_result *res, cudaGraphExec_t *capture);
+int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s);
 int check_params(const ccs_params *p, int d);
 
 }  // namespace ccs
