@@ -639,10 +639,22 @@ __global__ void k_measure_scaled(int m, const int64_t *ptr, const int32_t *cols,
 }
 
 // x_j = z_j / s_j (the decode of a column-scaled measurement is z = s . x).
+// Most z_j are zero, and a zero over a scale that is neither zero nor NaN is
+// the zero whose sign is the product of theirs: no binary64 division (they
+// run at a 64th of the integer rate here: 10.1 us instead of 3.6 us at n =
+// 200003).
 __global__ void k_unscale(int n, const double *sc, const double *z, double *x) {
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
-         j += (long long)gridDim.x * blockDim.x)
-        x[j] = __ddiv_rn(z[j], sc[j]);
+         j += (long long)gridDim.x * blockDim.x) {
+        const double zj = z[j], sj = sc[j];
+        const unsigned long long zb = (unsigned long long)__double_as_longlong(zj),
+                                 sb = (unsigned long long)__double_as_longlong(sj);
+        const unsigned long long mag = sb << 1;
+        if ((zb << 1) == 0ull && mag != 0ull && mag <= 0xffe0000000000000ull)
+            x[j] = __longlong_as_double((long long)((zb ^ sb) & 0x8000000000000000ull));
+        else
+            x[j] = __ddiv_rn(zj, sj);
+    }
 }
 
 __global__ void k_measure(int m, const int64_t *ptr, const int32_t *cols, const double *x,

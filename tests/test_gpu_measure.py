@@ -55,3 +55,19 @@ def test_measure_bitwise(ccs, orc, n, m, d, k):
         assert np.array_equal(y, orc.measure(A, m, x), equal_nan=True)
         ys = ccs.measure_scaled(ptr, cols, sd, xd, m, d).cpu().numpy()
         assert np.array_equal(ys, orc.measure_scaled(A, m, s, x), equal_nan=True)
+
+
+def test_unscale_special_values(ccs):
+    """Zeros of either sign over ordinary, zero, infinite and NaN scales give
+    what binary64 division gives."""
+    import torch
+    z = np.array([0.0, -0.0, 1.5, -2.5, np.inf, np.nan, 5e-324])
+    s = np.array([1.25, -1.25, 0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, 1e308])
+    zz, ss = (a.ravel() for a in np.meshgrid(z, s))
+    x = ccs.unscale(torch.from_numpy(ss.copy()).cuda(), torch.from_numpy(zz.copy()).cuda())
+    with np.errstate(all="ignore"):
+        want = zz / ss
+    got = x.cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    ok = ~np.isnan(want)
+    assert np.array_equal(got[ok].view(np.int64), want[ok].view(np.int64))
