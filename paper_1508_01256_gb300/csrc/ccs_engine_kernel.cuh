@@ -1250,10 +1250,13 @@ __device__ __forceinline__ long long residual_exact_tile(const ProblemDev &P, in
     return warp_sum_ll(delta);
 }
 
-// One row of the residual phase.  The touched flag, the row's slot record,
-// y_i and the old r_i are independent loads issued together; only touched
-// rows then gather their contributors' x_hat_j.
-// One row tile of the residual phase.  Rows with more contributors than
+// One row tile of the residual phase, a lane a row.  The touched flags come
+// first: most tiles of a late iteration have none set, and then the rows'
+// 64-byte records (8 MB at m = 2^17) stay where they are: 100 iterations at
+// n = 2^20, m = 2^17, d = 7 with two or three columns accepted in each take
+// 2314 us instead of 2374 us.  A touched row's
+// record, y_i and old r_i are independent loads issued together; its
+// contributors' x_hat_j follow.  Rows with more contributors than
 // their slot record holds are appended to the CTA's overflow list (summed
 // afterwards, one warp a row); when the list is full the warp sums them
 // itself.
@@ -1261,16 +1264,17 @@ static __device__ __noinline__ long long residual_tile(const ProblemDev &P, int 
                                                 int *ovf, int *ovf_n, int ovf_cap) {
     const int i = tile * kTile + lane;
     long long delta = 0;
-    bool touched = false, over = false;
+    const bool touched = i < P.m && __ldcg(P.touched + i) != 0;
+    if (!__any_sync(0xffffffffu, touched)) return 0;
+    bool over = false;
     int js[kSlotRec];
     double yi = 0.0, ro = 0.0, s = 0.0;
-    if (i < P.m) {
-        touched = __ldcg(P.touched + i) != 0;
+    if (touched) {
         load_record(P, i, js);
         yi = __ldg(P.y + i);
         ro = __ldcg(P.r + i);
-        over = touched && js[0] > kSlots;
-        if (touched && !over) s = row_sum_from_record(P, i, js);
+        over = js[0] > kSlots;
+        if (!over) s = row_sum_from_record(P, i, js);
     }
     bool later = false;
     if (over) {
