@@ -87,9 +87,9 @@ enum {
     CCS_ENGINE_AUTO = 0,       /* library's choice: problems small enough for
                                   one thread-block cluster's shared memory
                                   are decoded there (no grid barriers), the
-                                  others by the persistent engine; schedule
-                                  or debug_flags beyond bits 1-2 keep to the
-                                  persistent engine                          */
+                                  others, and a server's, by the persistent
+                                  engine; schedule or debug_flags beyond
+                                  bits 1-2 keep to the persistent engine     */
     CCS_ENGINE_HOST_LOOP = 1,  /* one launch per phase, host checks the stop
                                   rule after every iteration                 */
     CCS_ENGINE_PERSISTENT = 3  /* one cooperative launch runs every
@@ -316,11 +316,12 @@ CCS_API int ccs_decode_parallel_l0_async(int32_t n, int32_t m, int32_t d,
  * ccs_decode_batch -- Parallel-l0 on `count` independent problems of any
  * sizes in persistent cooperative launches (the iteration loop runs on the
  * device; each problem stops on its own rule and drops out of later
- * phases).  Problems small enough for a cluster (CCS_ENGINE_AUTO) go out in
- * one launch of their own.  Of the others, problems of one class (d <= 8 or d > 8; fingerprints of r in
- * shared memory or not) share a launch; when a batch holds several classes,
- * each class's launch runs a few iterations, then one launch over the whole
- * batch continues the problems still running.  Per problem, the results are
+ * phases).  When a third of the problems or more are small enough for a
+ * cluster (CCS_ENGINE_AUTO), those go out in one launch of their own.  Of the
+ * others, problems of one class (d <= 8 or d > 8; fingerprints of r in shared
+ * memory or not) share a launch; when they are of several classes, each
+ * class's launch runs a few iterations, then one launch over all of them
+ * continues the problems still running.  Per problem, the results are
  * bit-identical to ccs_decode_parallel_l0 on that problem alone.
  *
  * probs: host array of `count` descriptors (device pointers inside);

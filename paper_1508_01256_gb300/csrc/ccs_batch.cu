@@ -182,19 +182,34 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
         }
         return CCS_OK;
     }
-    // Problems that fit a cluster on chip go out in one launch of the small
-    // engine.  The others go out as up to four launches, one per class, each
-    // over the whole GPU: d <= 8 and d > 8 run on different kernel instances
-    // (the register-resident arrays are sized by the largest d of a launch),
-    // and problems whose fingerprints do not fit shared memory would shrink
+    // When a third of the problems or more fit a cluster on chip, those go out
+    // in one launch of the small engine.  The problems that run to max_iter
+    // decide the time of a batch: their iterations take 5-23 us there
+    // against ~16 us shared by all problems in the persistent engine, which
+    // has to run them anyway once one of the larger problems does not
+    // converge.  Measured, small engine against none: 39 of 44 problems fit
+    // 1.53 against 2.82 ms, 36 of 62 1.50 / 3.60, 29 of 64 2.36 / 4.51, 10 of
+    // 27 2.25 / 2.92; below a third 5 of 21 0.72 / 0.70, 7 of 41 6.57 / 6.02,
+    // 3 of 63 5.95 / 5.15.  Sending only the smaller ones of them (by n d, by
+    // m) gave the worse of both.
+    //
+    // The others go out as up to four launches, one per class, each over the
+    // whole GPU: d <= 8 and d > 8 run on different kernel instances (the
+    // register-resident arrays are sized by the largest d of a launch), and
+    // problems whose fingerprints do not fit shared memory would shrink
     // every other problem's launch plan (fewer stages, a smaller queue) and
     // its thread count.  Every problem's result is the same either way.
     constexpr int kSmallClass = 4;
-    std::vector<int> cls(count);
+    std::vector<int> cls(count, -1);
+    int on_chip = 0;
+    for (int32_t q = 0; q < count && !tuned; ++q)
+        if (small_route(pds[q], p, count == 1)) {
+            cls[q] = kSmallClass;
+            ++on_chip;
+        }
     for (int32_t q = 0; q < count; ++q)
-        cls[q] = !tuned && small_route(pds[q], p, count == 1)
-                     ? kSmallClass
-                     : (pds[q].d > 8 ? 2 : 0) + (engine_fp_fits(pds[q], p) ? 0 : 1);
+        if (cls[q] < 0 || 3 * on_chip < count)
+            cls[q] = (pds[q].d > 8 ? 2 : 0) + (engine_fp_fits(pds[q], p) ? 0 : 1);
     // descriptors in launch order; out_slot keeps the caller's index
     std::vector<ProblemDev> sub;
     int sizes[4] = {0, 0, 0, 0};

@@ -346,7 +346,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     }
 
     if (small) {
-        if ((rc = small_launch(pds, nullptr, 1, prm, false, 0x7fffffff, a.sync, dev_out, s,
+        if ((rc = small_launch(pds, nullptr, 1, prm, a.sync, dev_out, s,
                                true)))
             return rc;
     } else {
@@ -500,7 +500,7 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
         int rc;
         if (rest < count &&
             (rc = small_launch(pds + rest, count > 1 ? d_fresh + rest : nullptr, count - rest, prm,
-                               false, 0x7fffffff, sync, res, cs, !capture)))
+                               sync, res, cs, !capture)))
             return rc;
         for (int l = 0; l < launches; ++l) {
             const LaunchPlan &L = plans[l];
@@ -552,40 +552,29 @@ int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s) {
     return CCS_OK;
 }
 
-// A server round.  Problems that fit a cluster on chip go out in a launch of
-// their own.  pds: out_slot 0..P-1, in any order.
+// A server round: one resume-mode launch.
 int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
                   char *hdr, cudaStream_t s) {
-    const int rest = (int)(std::stable_partition(pds, pds + P, [&](const ProblemDev &q) {
-                               return !small_route(q, prm, P == 1);
-                           }) - pds);
-    EngineSync *sync = reinterpret_cast<EngineSync *>(hdr);
-    ccs_result *res = reinterpret_cast<ccs_result *>(hdr + sizeof(EngineSync));
+    LaunchPlan L;
+    int rc = plan_launch(pds, P, prm, L);
+    if (rc) return rc;
     ProblemDev *d_probs =
         reinterpret_cast<ProblemDev *>(hdr + resume_results_bytes(P) + stamps_bytes());
-    LaunchPlan L{};
-    int rc;
-    if (rest && (rc = plan_launch(pds, rest, prm, L))) return rc;
-    CCS_CUDA_TRY(cudaMemsetAsync(sync, 0, sizeof(EngineSync), s));
+    EngineArgs a;
+    fill_args(a, L, P, prm);
+    a.resume = 1;
+    a.iter_budget = iter_budget > 0 ? iter_budget : 1;
+    a.sync = reinterpret_cast<EngineSync *>(hdr);
+    a.dev_out = reinterpret_cast<ccs_result *>(hdr + sizeof(EngineSync));
+    a.probs = d_probs;
+    CCS_CUDA_TRY(cudaMemsetAsync(hdr, 0, sizeof(EngineSync), s));
     CCS_CUDA_TRY(cudaMemcpyAsync(d_probs, pds, sizeof(ProblemDev) * P, cudaMemcpyHostToDevice, s));
-    if (rest < P && (rc = small_launch(pds + rest, d_probs + rest, P - rest, prm, true,
-                                       iter_budget, sync, res, s, true)))
-        return rc;
-    if (rest) {
-        EngineArgs a;
-        fill_args(a, L, rest, prm);
-        a.resume = 1;
-        a.iter_budget = iter_budget > 0 ? iter_budget : 1;
-        a.sync = sync;
-        a.dev_out = res;
-        a.probs = d_probs;
-        void *args[] = {&a};
-        const int ev = prof_start(CCS_K_PERSISTENT, s);
-        CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads),
-                                                 args, L.smem, s));
-        prof_stop(ev, s);
-        count_launches(1);
-    }
+    void *args[] = {&a};
+    const int ev = prof_start(CCS_K_PERSISTENT, s);
+    CCS_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)L.fn, dim3(L.G), dim3(L.threads), args,
+                                             L.smem, s));
+    prof_stop(ev, s);
+    count_launches(1);
     return engine_results(hdr, P, out, s);
 }
 

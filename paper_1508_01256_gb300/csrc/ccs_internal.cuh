@@ -208,7 +208,7 @@ size_t engine_resume_header_bytes(int P);
 // (alone: nothing else shares the GPU with it).
 bool small_route(const ProblemDev &pd, const ccs_params &prm, bool alone);
 int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_params &prm,
-                 bool resume, int iter_budget, EngineSync *sync, ccs_result *dev_out,
+                 EngineSync *sync, ccs_result *dev_out,
                  cudaStream_t s, bool timed);
 
 // The expander's construction (ccs_setup.cu): all of it enqueued, then what

@@ -18,7 +18,10 @@
 // stay in global memory; few columns are accepted.
 //
 // Clusters take the problems of a launch one after another, so a batch's
-// small problems run side by side, each at its own pace.  The method, its
+// small problems run side by side, each at its own pace (a server's rounds of
+// two iterations stay with the engine: loading a problem's rows each round
+// cost what it gave, 17 problems of n = 10000-30000 1.55 ms against 1.45, 24
+// of n = 4096-500000 7.1-8.1 ms against 7.1-7.8).  The method, its
 // order of operations and the residual forms are the engine's (see there):
 // results are the same bits.
 //
@@ -61,8 +64,6 @@ struct SmallArgs {
     const ProblemDev *probs;
     int P;
     int alpha, mode, max_iter, debug_flags, shifted;
-    int resume;                // only kPdFresh problems start; the others continue
-    int iter_budget;
     EngineSync *sync;
     ccs_result *dev_out;       // or null
 };
@@ -217,11 +218,10 @@ struct SmallState {
     unsigned long long all_xnew[2][kSmallCluster];
 };
 
-// One problem by the cluster: from its first (or next) iteration to its end or
-// the launch's iteration budget.
+// One problem by the cluster, from its first iteration to its end.
 template <int DMAX>
 __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDev &P, SmallState &s,
-                                             char *smem, bool fresh) {
+                                             char *smem) {
     const cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -233,7 +233,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
     SmallSmem S;
     small_smem(n, m, d, C, smem, &S);
 
-    // ---- state on chip; Alg. 2, first line, for a fresh problem ---------
+    // ---- state on chip; Alg. 2, first line ------------------------------
     if (tid == 0) {
         s.r0 = 0;
         s.rmax = 0;
@@ -251,7 +251,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
     int nz = 0, gridb = 0, deg = 0;
     unsigned long long mx = 0;
     for (int i = tid; i < m; i += kSmallThreads) {
-        const double v = fresh ? __ldg(P.y + i) : __ldcg(P.r + i);
+        const double v = __ldg(P.y + i);
         const unsigned long long b = value_bits(v);
         S.r[i] = v;
         S.delta[i] = S.delta[m + i] = 0.0;
@@ -260,14 +260,11 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
         const unsigned long long mag = b & 0x7fffffffffffffffull;
         nz += mag != 0;
         mx = mag > mx ? mag : mx;
-        if (fresh) {
-            if (mag) gridb = max(gridb, 1100 - lowbit_exponent(mag));
-            deg = max(deg, (int)(__ldg(P.csr_ptr + i + 1) - __ldg(P.csr_ptr + i)));
-            if (i % C == rank) P.slots[(size_t)i * kSlotRec] = 0;
-        }
+        if (mag) gridb = max(gridb, 1100 - lowbit_exponent(mag));
+        deg = max(deg, (int)(__ldg(P.csr_ptr + i + 1) - __ldg(P.csr_ptr + i)));
+        if (i % C == rank) P.slots[(size_t)i * kSlotRec] = 0;
     }
-    if (fresh)
-        for (int j = tid; j < cols; j += kSmallThreads) P.x_hat[c0 + j] = 0.0;
+    for (int j = tid; j < cols; j += kSmallThreads) P.x_hat[c0 + j] = 0.0;
     nz = __reduce_add_sync(0xffffffffu, nz);
     mx = warp_max_bits(mx);
     gridb = __reduce_max_sync(0xffffffffu, gridb);
@@ -280,27 +277,11 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
     }
     __syncthreads();
     if (tid == 0) {
-        if (fresh) {
-            s.it = s.empty_run = s.rmode = 0;
-            s.xmax = 0;
-            s.status = s.r0 == 0 ? CCS_CONVERGED
-                                 : (a.max_iter == 0 ? CCS_MAX_ITER : kRunning);
-            s.cert = certificate_from(s.gridb, s.rmax, s.deg);
-            if (rank == 0) {
-                ctrl->grid_b = s.gridb;
-                ctrl->ymax = s.rmax;
-                ctrl->deg = s.deg;
-                if (P.r0_hist) P.r0_hist[0] = s.r0;
-            }
-        } else {
-            s.it = __ldcg(&ctrl->iteration);
-            s.empty_run = ctrl->empty_run[s.it & 1];
-            s.rmode = __ldcg(&ctrl->ordered) ? 1 : 0;
-            s.xmax = __ldcg(&ctrl->xmax[0]);
-            s.status = kRunning;
-            s.cert = certificate_from(__ldcg(&ctrl->grid_b), __ldcg(&ctrl->ymax),
-                                          __ldcg(&ctrl->deg));
-        }
+        s.it = s.empty_run = s.rmode = 0;
+        s.xmax = 0;
+        s.status = s.r0 == 0 ? CCS_CONVERGED : (a.max_iter == 0 ? CCS_MAX_ITER : kRunning);
+        s.cert = certificate_from(s.gridb, s.rmax, s.deg);
+        if (rank == 0 && P.r0_hist) P.r0_hist[0] = s.r0;
     }
     // Thread 0: the residual form of the next iteration.
     auto next_form = [&]() {
@@ -312,7 +293,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
     if (tid == 0 && s.status == kRunning) next_form();
     cl.sync();  // every CTA's copy is ready for the others' updates
 
-    for (int g = 0; g < a.iter_budget && s.status == kRunning; ++g) {
+    while (s.status == kRunning) {
         const int it = s.it, par = it & 1;
         double *const delta = S.delta + (par ? m : 0);
         uint8_t *const touched = S.touched + (par ? m : 0);
@@ -535,7 +516,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
                 s.status = s.r0 == 0 ? CCS_CONVERGED
                                      : (it + 1 >= a.max_iter ? CCS_MAX_ITER : kRunning);
                 if (rank == 0 && P.r0_hist) P.r0_hist[it + 1] = s.r0;
-                if (s.status == kRunning && g + 1 < a.iter_budget) next_form();
+                if (s.status == kRunning) next_form();
             }
         }
         __syncthreads();
@@ -549,8 +530,6 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
         ctrl->iteration = s.it;
         ctrl->r0 = s.r0;
         ctrl->ordered = s.rmode != 0;
-        ctrl->xmax[0] = s.xmax;
-        ctrl->empty_run[s.it & 1] = (short)s.empty_run;
     }
 }
 
@@ -574,21 +553,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
         if (s.problem < 0) break;
         if (threadIdx.x == 0) P = a.probs ? a.probs[s.problem] : a.single;
         __syncthreads();
-        const bool fresh = !a.resume || (P.flags & kPdFresh);
-        const bool runs = fresh || __ldcg(&P.ctrl->status) == kRunning;  // same in every CTA
-        if (!runs) {
-            cl.sync();  // every CTA knows the problem before the next one is taken
-        } else if (P.d <= 5) {
-            small_decode<5>(a, P, s, smem, fresh);
-        } else if (P.d <= 7) {
-            small_decode<7>(a, P, s, smem, fresh);
-        } else if (P.d <= 9) {
-            small_decode<9>(a, P, s, smem, fresh);
-        } else if (P.d <= 12) {
-            small_decode<12>(a, P, s, smem, fresh);
-        } else {
-            small_decode<16>(a, P, s, smem, fresh);
-        }
+        if (P.d <= 5) small_decode<5>(a, P, s, smem);
+        else if (P.d <= 7) small_decode<7>(a, P, s, smem);
+        else if (P.d <= 9) small_decode<9>(a, P, s, smem);
+        else if (P.d <= 12) small_decode<12>(a, P, s, smem);
+        else small_decode<16>(a, P, s, smem);
         if (leader && a.dev_out) {
             const DecodeCtrl *c = P.ctrl;
             ccs_result res;
@@ -660,9 +629,9 @@ static int small_clusters(int dev, int C) {
 // P problems (descriptors `pds` on the host; `dev` the same ones in device
 // memory, or null for a single one), enqueued on `s` (`timed`: with the
 // profiler's events, which a capture leaves out).  The sync word's
-// `next` and the fresh problems' control blocks start at zero.
+// `next` starts at zero.
 int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_params &prm,
-                 bool resume, int iter_budget, EngineSync *sync, ccs_result *dev_out,
+                 EngineSync *sync, ccs_result *dev_out,
                  cudaStream_t s, bool timed) {
     long long entries = 0;
     for (int p = 0; p < P; ++p) {
@@ -691,8 +660,6 @@ int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_
     a.max_iter = prm.max_iter;
     a.debug_flags = prm.debug_flags;
     a.shifted = prm.shifted;
-    a.resume = resume;
-    a.iter_budget = iter_budget > 0 ? iter_budget : 1;
     a.sync = sync;
     a.dev_out = dev_out;
     cudaLaunchConfig_t cfg{};

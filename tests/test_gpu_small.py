@@ -103,3 +103,14 @@ def test_batch_of_small_and_large_problems(ccs, orc):
         assert np.array_equal(x_hat.cpu().numpy(), ref["x_hat"])
         assert np.array_equal(r.cpu().numpy(), ref["r"])
     graph.close()
+
+
+@pytest.mark.parametrize("small, large", [(1, 3), (1, 2), (2, 2)])
+def test_batch_on_both_sides_of_the_rule(ccs, orc, small, large):
+    """The small engine takes a batch's small problems when they are a third of it."""
+    probs = [_problem(c)[0] for c in ("ragged_parts", "oscillates")[:small]]
+    probs += [inputs.make_problem(120001, 12001, 7, 1500, 5), inputs.make_problem(130001, 1300, 9, 90, 6),
+              inputs.make_problem(140001, 1400, 7, 140, 7)][:large]
+    for g, p in zip(ccs.decode_batch([device_problem(ccs, p) for p in probs], history=True), probs):
+        A, y_ref = oracle_problem(orc, p)
+        assert_same_decode(g, orc.parallel_l0(A, p.m, y_ref))
