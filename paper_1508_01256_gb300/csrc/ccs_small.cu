@@ -11,9 +11,11 @@
 //   - every CTA holds all of r, its fingerprints, the changes of this
 //     iteration and the touched flags; an accepted column updates all the
 //     cluster's copies (distributed shared memory);
-//   - one hardware cluster barrier an iteration (two under the ordered
-//     residual, whose row sums are shared out): every CTA then brings its copy
-//     of r up to date and evaluates the stop rule by itself.
+//   - one hardware cluster barrier an iteration, one more under the ordered
+//     residual, whose row sums are shared out, and one more when a CTA accepts
+//     more columns than its list holds: every CTA then brings its copy of r up
+//     to date and evaluates the stop rule by itself, so all copies have to end
+//     with the same bits.
 // x_hat, the contributor records of the ordered residual and the CSR rows
 // stay in global memory; few columns are accepted.
 //
@@ -436,14 +438,18 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
                     if (exact) sum = __dadd_rn(sum, *cl.map_shared_rank(delta + i, q));
                     hit |= *cl.map_shared_rank(touched + i, q);
                 }
-                delta_next[i] = sum;
+                if (exact) delta_next[i] = sum;
                 touched_next[i] = hit;
             }
             cl.sync();
             for (int i = tid; i < m; i += kSmallThreads) {
-                delta[i] = __dadd_rn(delta[i], delta_next[i]);
+                // under the ordered residual `delta` belongs from here on to
+                // the CTA that sums row i, which may already be storing to it
+                if (exact) {
+                    delta[i] = __dadd_rn(delta[i], delta_next[i]);
+                    delta_next[i] = 0.0;
+                }
                 touched[i] |= touched_next[i];
-                delta_next[i] = 0.0;
                 touched_next[i] = 0;
             }
         }
