@@ -544,16 +544,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
     __shared__ ProblemDev P;
     __shared__ SmallState s;
     const cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks();
     const bool leader = cl.block_rank() == 0 && threadIdx.x == 0;
+    // another CTA's shared memory may be written once that CTA runs
+    if (a.probs) cl.sync();
     for (bool first = true;; first = false) {
-        if (leader) {  // the cluster's next problem
-            int p = first ? 0 : -1;
-            if (a.probs) {
-                const unsigned k = atomicAdd(&a.sync->next, 1u);
-                p = k < (unsigned)a.P ? (int)k : -1;
-            }
-            for (int q = 0; q < C; ++q) *cl.map_shared_rank(&s.problem, q) = p;
+        if (!a.probs) {  // one problem: every CTA knows
+            if (threadIdx.x == 0) s.problem = first ? 0 : -1;
+        } else if (leader) {  // the cluster's next problem
+            const unsigned k = atomicAdd(&a.sync->next, 1u);
+            const int p = k < (unsigned)a.P ? (int)k : -1;
+            for (int q = 0; q < (int)cl.num_blocks(); ++q) *cl.map_shared_rank(&s.problem, q) = p;
         }
         cl.sync();  // also: every CTA is done with the previous problem
         if (s.problem < 0) break;

@@ -8,7 +8,8 @@ more contributors than their records hold."""
 import numpy as np
 import pytest
 
-from gpu_util import assert_same_decode, upload_matrix
+from gpu_util import assert_same_decode, device_problem, oracle_problem, upload_matrix
+from paper_1508_01256_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -101,3 +102,38 @@ def test_batch_with_long_lists(ccs, orc, flags):
             items.append((*upload_matrix(orc, A, m), torch.from_numpy(y).cuda()))
     for g, ref in zip(ccs.decode_batch(items, max_iter=25, history=True, debug_flags=flags), refs):
         assert_same_decode(g, ref)
+
+
+def test_clusters_that_start_at_different_times(ccs, orc):
+    """Batches of small problems on two streams beside decodes that fill the
+    GPU: a cluster's CTAs start as SMs become free, each problem once and
+    with its own results."""
+    import torch
+    probs = [inputs.make_problem(60001, 6000, 7, 600, 5)]
+    probs += [inputs.make_problem(3001 + 997 * q, 400 + 60 * q, 7, 30 + 6 * q, 60 + q) for q in range(6)]
+    items = [device_problem(ccs, p) for p in probs]
+    refs = []
+    for p in probs:
+        A, y = oracle_problem(orc, p)
+        refs.append(orc.parallel_l0(A, p.m, y))
+
+    def outputs(chosen):
+        return [(torch.full((probs[q].n,), float("nan"), dtype=torch.float64, device="cuda"),
+                 torch.empty(probs[q].m, dtype=torch.float64, device="cuda")) for q in chosen]
+
+    lanes = []
+    for chosen in ([0], range(1, 7), range(1, 7)):
+        bufs = outputs(chosen)
+        pbs = [ccs.problem(*items[q], *b) for q, b in zip(chosen, bufs)]
+        lanes.append((list(chosen), bufs, pbs, ccs.BatchGraph(pbs), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for _, _, _, graph, stream in lanes:
+            graph.launch(stream)
+    torch.cuda.synchronize()
+    for chosen, bufs, _, graph, _ in lanes:
+        for q, (x, _), res in zip(chosen, bufs, graph.read_results()):
+            assert (res.status, res.iterations, res.error) == \
+                (refs[q]["status"], refs[q]["iterations"], 0)
+            assert np.array_equal(x.cpu().numpy(), refs[q]["x_hat"])
+        graph.close()
