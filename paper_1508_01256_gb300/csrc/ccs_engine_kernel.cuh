@@ -1204,7 +1204,8 @@ __device__ __noinline__ void row_hits_clear(const ProblemDev &P) {
 // (a row's partial sums of x_hat, and r_i minus the omegas accepted in its
 // row during the iteration).  The test below asks for that bound to stay
 // under 2^(e+51), a factor 4 below the limit, which covers the rounding of
-// the bound's own evaluation.  Every CTA evaluates it from the same stored
+// the bound's own evaluation, and under 2^1023, so that no partial sum
+// overflows in any order.  Every CTA evaluates it from the same stored
 // maxima (written before the previous grid barrier), so all agree.
 __device__ __forceinline__ bool exact_certified(const DecodeCtrl *c, int it, int debug_flags) {
     if ((debug_flags & kFlagOrdered) || ((debug_flags & kFlagSwitch) && it >= 2)) return false;
@@ -1215,8 +1216,7 @@ __device__ __forceinline__ bool exact_certified(const DecodeCtrl *c, int it, int
     const double R = __longlong_as_double((long long)__ldcg(&c->rmax[it & 1]));
     const double X = __longlong_as_double((long long)__ldcg(&c->xmax[it & 1]));
     const double bound = Y + (double)__ldcg(&c->deg) * (X + 2.0 * R);
-    if (e + 51 > 1023) return true;
-    return bound < ldexp(1.0, e + 51);
+    return bound < ldexp(1.0, min(e + 51, 1023));
 }
 
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {

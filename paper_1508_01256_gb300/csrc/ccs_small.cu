@@ -168,9 +168,11 @@ __device__ __forceinline__ bool score_pairs(const unsigned long long (&v)[DMAX],
 }
 
 // The exactness certificate of the incremental residual, as in the engine:
-// while Y + deg (X + 2 R) < 2^(e+51), with Y, X, R the largest |y_i|,
-// |x_hat_j|, |r_i| and e the exponent of the lowest set bit over the nonzero
-// y_i, every addition of the iteration is exact.
+// while Y + deg (X + 2 R) < 2^min(e+51, 1023), with Y, X, R the largest
+// |y_i|, |x_hat_j|, |r_i| and e the exponent of the lowest set bit over the
+// nonzero y_i, every addition of the iteration is exact and none overflows.
+// (A sum that overflows in one order and not in another would leave the
+// CTAs' copies of r different.)
 struct Certificate {
     double Y, deg, limit;  // limit < 0: always holds
 };
@@ -181,8 +183,8 @@ __device__ __forceinline__ Certificate certificate_from(int grid_b, unsigned lon
     Certificate q;
     q.Y = __longlong_as_double((long long)ymax);
     q.deg = (double)deg;
-    // y == 0 (nothing is ever added), or a limit beyond every double
-    q.limit = (grid_b == 0 || e + 51 > 1023) ? -1.0 : ldexp(1.0, e + 51);
+    // y == 0: nothing is ever added
+    q.limit = grid_b == 0 ? -1.0 : ldexp(1.0, min(e + 51, 1023));
     return q;
 }
 
