@@ -129,10 +129,10 @@ static DeviceInfo device_info(int dev) {
 // device's opt-in limit per CTA minus the kernel's static shared memory.
 // The kernel's attribute is raised to it once, so every later launch of any
 // size up to it is allowed.  Returns 0 on failure.
-static size_t max_dynamic_smem(int dev, engine_fn fn) {
+size_t max_dynamic_smem(int dev, const void *fn) {
     struct Entry {
         int dev;
-        engine_fn fn;
+        const void *fn;
         size_t lim;
     };
     static std::mutex mu;
@@ -213,7 +213,7 @@ static int plan_launch(ProblemDev *pds, int P, const ccs_params &prm, LaunchPlan
     const int warps = threads / 32;
     int dev = 0;
     CCS_CUDA_TRY(cudaGetDevice(&dev));
-    const size_t smem_limit = max_dynamic_smem(dev, fn);
+    const size_t smem_limit = max_dynamic_smem(dev, (const void *)fn);
     if (smem_limit == 0) {
         set_last_error("could not size the engine's shared memory");
         return CCS_ECUDA;
@@ -304,7 +304,7 @@ bool engine_fp_fits(const ProblemDev &pd, const ccs_params &prm) {
     engine_fn fn = engine_kernel(pd.d, sched);
     int dev = 0;
     if (!fn || cudaGetDevice(&dev) != cudaSuccess) return false;
-    const size_t smem_limit = max_dynamic_smem(dev, fn);
+    const size_t smem_limit = max_dynamic_smem(dev, (const void *)fn);
     const int threads = sched == 1 ? 1024 : (sched == 3 ? 768 : 512);
     const int tpw = sched == 2 ? 2 : 1;
     const size_t stage_bytes = align_up((size_t)(threads / 32 - 1) * tpw * kTile * pd.d * 4, 128);

@@ -203,6 +203,10 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
 // iter_budget iterations run; out[p].status is -1 for problems still
 // running.  `hdr` needs engine_resume_header_bytes(P) bytes.
 size_t engine_resume_header_bytes(int P);
+// Largest dynamic shared memory a launch of kernel `fn` may use on `dev`, the
+// kernel's attribute raised to it (ccs_engine.cu); 0 on failure.
+size_t max_dynamic_smem(int dev, const void *fn);
+
 // Small problems (ccs_small.cu): decoded by one thread-block cluster each, on
 // chip.  small_route: whether a problem takes that path under these params
 // (alone: nothing else shares the GPU with it).

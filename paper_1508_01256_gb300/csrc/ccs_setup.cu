@@ -1037,6 +1037,17 @@ static ExpanderWs expander_ws(int32_t m, void *ws) {
     return w;
 }
 
+// Lets launches of `fn` use `bytes` of shared memory.  The attribute belongs to
+// the kernel, not to the call: it is raised to the device's limit and never
+// lowered, so threads drawing matrices of different sizes do not meet.
+static int allow_smem(const void *fn, size_t bytes) {
+    int dev = 0;
+    CCS_CUDA_TRY(cudaGetDevice(&dev));
+    if (max_dynamic_smem(dev, fn) >= bytes) return CCS_OK;
+    set_last_error("ccs_make_expander: a kernel cannot use %zu bytes of shared memory", bytes);
+    return CCS_ECUDA;
+}
+
 // The whole construction, for one d.
 template <int D>
 static int expander_build(int32_t n, int32_t m, uint64_t seed, int32_t *csc_rows,
@@ -1045,10 +1056,11 @@ static int expander_build(int32_t n, int32_t m, uint64_t seed, int32_t *csc_rows
     const long long edges = (long long)n * D;
     CCS_CUDA_TRY(cudaMemsetAsync(w.deg, 0, w.bytes, s));
     if (pl.groups) {
-        const auto big = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        CCS_CUDA_TRY(cudaFuncSetAttribute(k_draw_columns<D>, big, (int)pl.draw_smem));
-        CCS_CUDA_TRY(cudaFuncSetAttribute(k_deal_entries<D>, big, (int)pl.deal_smem));
-        CCS_CUDA_TRY(cudaFuncSetAttribute(k_sort_groups, big, (int)pl.sort_smem));
+        int rc;
+        if ((rc = allow_smem((const void *)k_draw_columns<D>, pl.draw_smem)) ||
+            (rc = allow_smem((const void *)k_deal_entries<D>, pl.deal_smem)) ||
+            (rc = allow_smem((const void *)k_sort_groups, pl.sort_smem)))
+            return rc;
         const int draw_grid = (int)std::min(((long long)n + kDrawBlock - 1) / kDrawBlock, 3ll * pl.sms);
         k_draw_columns<D><<<draw_grid, kDrawBlock, pl.draw_smem, s>>>(n, m, seed, pl.row_bits,
                                                                      pl.groups, csc_rows, w.deg);
