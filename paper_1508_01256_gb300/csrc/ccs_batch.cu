@@ -139,10 +139,6 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
                                        pr.r, pr.r0_hist)))
             return rc;
     }
-    if (count > kMaxBatch) {
-        set_last_error("at most %d problems per launch (got %d)", kMaxBatch, count);
-        return CCS_EINVAL;
-    }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     char *hdr = static_cast<char *>(ws);
     char *rhdr = hdr + engine_header_bytes(count);
@@ -181,6 +177,11 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
             if (rc != CCS_OK) return rc;
         }
         return CCS_OK;
+    }
+    // the autotuner runs the launch groups one by one, each within the limit
+    if (count > kMaxBatch && !tuned) {
+        set_last_error("at most %d problems per launch (got %d)", kMaxBatch, count);
+        return CCS_EINVAL;
     }
     // When a third of the problems or more fit a cluster on chip, those go out
     // in one launch of the small engine.  The problems that run to max_iter
