@@ -241,7 +241,13 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
     if ((rc = engine_run_batch(sub.data(), sizes, groups, count, p, kGroupIters, hdr, rhdr, s, res,
                                capture)))
         return rc;
-    return dev_out ? CCS_OK : engine_results(rhdr, count, out, s);
+    if (dev_out) return CCS_OK;
+    rc = engine_results(rhdr, count, out, s);
+    if (rc == CCS_ETIMEOUT) {
+        const int rc2 = engine_stopped_results(sub.data(), count, hdr, out);
+        if (rc2) return rc2;
+    }
+    return rc;
 }
 
 extern "C" int ccs_decode_batch(const ccs_problem *probs, int32_t count, const ccs_params *params,

@@ -315,6 +315,17 @@ bool engine_fp_fits(const ProblemDev &pd, const ccs_params &prm) {
     return need <= smem_limit - fixed - 2 * stage_bytes;
 }
 
+static void result_of(const DecodeCtrl &c, bool timed_out, ccs_result &out) {
+    out.status = c.status;
+    out.iterations = c.iteration;
+    out.r0_final = c.r0;
+    out.error = timed_out ? CCS_ETIMEOUT : CCS_OK;
+    out.row_driven = c.row_driven;
+    out.row_entries = c.row_entries;
+    out.residual_form = c.ordered ? CCS_RESIDUAL_ORDERED : CCS_RESIDUAL_EXACT;
+    out.reserved = 0;
+}
+
 int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, char *ws,
                cudaStream_t s, ccs_result *dev_out) {
     const bool small = P == 1 && small_route(pds[0], prm, true);
@@ -384,14 +395,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     for (int p = 0; p < P; ++p) {
         DecodeCtrl hc;
         std::memcpy(&hc, hdr + sizeof(EngineSync) + sizeof(DecodeCtrl) * (size_t)p, sizeof(hc));
-        out[p].status = hc.status;
-        out[p].iterations = hc.iteration;
-        out[p].r0_final = hc.r0;
-        out[p].error = herr ? CCS_ETIMEOUT : CCS_OK;
-        out[p].row_driven = hc.row_driven;
-        out[p].row_entries = hc.row_entries;
-        out[p].residual_form = hc.ordered ? CCS_RESIDUAL_ORDERED : CCS_RESIDUAL_EXACT;
-        out[p].reserved = 0;
+        result_of(hc, herr != 0, out[p]);
         max_it = std::max(max_it, hc.iteration);
     }
     if (a.stamps) prof_keep_stamps(hst.data(), (int)hst.size(), kSubBase);
@@ -549,6 +553,16 @@ int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s) {
         set_last_error("a bounded device wait exceeded the watchdog");
         return CCS_ETIMEOUT;
     }
+    return CCS_OK;
+}
+
+// Results of a batch whose launch timed out before it wrote them: each
+// problem as its control block stands.
+int engine_stopped_results(const ProblemDev *pds, int P, char *hdr, ccs_result *out) {
+    std::vector<DecodeCtrl> c(P);
+    CCS_CUDA_TRY(cudaMemcpy(c.data(), header_ctrl(hdr, 0), sizeof(DecodeCtrl) * (size_t)P,
+                            cudaMemcpyDeviceToHost));
+    for (int t = 0; t < P; ++t) result_of(c[t], true, out[pds[t].out_slot]);
     return CCS_OK;
 }
 

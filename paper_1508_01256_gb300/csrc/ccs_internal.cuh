@@ -232,6 +232,7 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
                      const ccs_params &prm, int group_iters, char *hdr, char *rhdr,
                      cudaStream_t s, ccs_result *res, cudaGraphExec_t *capture);
 int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s);
+int engine_stopped_results(const ProblemDev *pds, int P, char *hdr, ccs_result *out);
 int check_params(const ccs_params *p, int d);
 
 }  // namespace ccs

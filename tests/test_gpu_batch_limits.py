@@ -1,5 +1,7 @@
 """Batches at and beyond the launch limits: more problems than one launch of
-the persistent engine takes."""
+the persistent engine takes, and a batch whose bounded waits run out."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -60,3 +62,26 @@ def test_more_problems_than_a_launch(ccs, orc):
         assert sum(t != 0 for t in ccs.ccs_autotune(pbs, ccs.params(), ws)) == 2
     finally:
         ccs.ccs_autotune_reset()
+
+
+def test_batch_that_times_out_reports_where_it_stood(ccs):
+    """CTA 0 never arrives at the first score barrier (test hook), so every
+    bounded wait runs out; each problem reports the time-out and the state
+    it was in: no iteration done, ||r||_0 of y."""
+    import torch
+    probs = [inputs.make_problem(5003, 500, 7, 20, 8), inputs.make_problem(6007, 600, 5, 30, 9)]
+    items = [device_problem(ccs, p) for p in probs]
+    pbs = [ccs.problem(*it, torch.empty(p.n, dtype=torch.float64, device="cuda"),
+                       torch.empty(p.m, dtype=torch.float64, device="cuda"))
+           for it, p in zip(items, probs)]
+    ws = ccs.workspace(ccs.ccs_batch_workspace_size(pbs))
+    ws.fill_(0x55)
+    torch.cuda.synchronize()
+    arr = (ccs.Problem * 2)(*pbs)
+    out = (ccs.Result * 2)()
+    prm = ccs.params(engine=ccs.ENGINE_PERSISTENT, watchdog_ms=200, debug_flags=1)
+    rc = ccs.lib().ccs_decode_batch(arr, 2, ctypes.byref(prm), out, ws.data_ptr(), ws.numel(), None)
+    assert rc == ccs.CCS_ETIMEOUT
+    for (_, _, _, y), res in zip(items, out):
+        assert (res.status, res.iterations, res.error) == (-1, 0, ccs.CCS_ETIMEOUT)
+        assert res.r0_final == int((y != 0).sum())
