@@ -542,11 +542,14 @@ enum {
     CCS_K_SCORE = 1,       /* score + apply (all columns)                   */
     CCS_K_RESIDUAL = 2,    /* r on touched rows + ||r||_0                    */
     CCS_K_FINISH = 3,      /* stop rule                                      */
-    CCS_K_PERSISTENT = 4,  /* whole decode in one cooperative launch; its
-                              score and residual phases are also reported
-                              under CCS_K_SCORE / CCS_K_RESIDUAL (device
-                              timer between grid barriers, one entry per
-                              iteration)                                    */
+    CCS_K_PERSISTENT = 4,  /* whole decode in one launch (cooperative, or of
+                              thread-block clusters); after a blocking call
+                              that makes one such launch its score and
+                              residual phases are also reported under
+                              CCS_K_SCORE / CCS_K_RESIDUAL (device timer
+                              between barriers, one entry per iteration; of
+                              a batch decoded by clusters, the iterations of
+                              its largest problem)                          */
     CCS_K_PHASE_FP = 5,     /* score phase seen from CTA 0: wait for the
                               residual fingerprints                         */
     CCS_K_PHASE_STREAM = 6, /* ... stream of the CSC through the fingerprint
@@ -562,11 +565,12 @@ typedef struct {
 CCS_API int ccs_profile_begin(void);
 /* times: array of CCS_K_COUNT entries (host). */
 CCS_API int ccs_profile_end(ccs_kernel_time *times);
-/* Phase times of one iteration of the last persistent launch made while
- * profiling (device timer between grid barriers): phase_us[0] score phase,
- * [1] residual phase, [2..4] CTA 0's score sub-phases (fingerprints in,
- * stream, queued candidates; -1 when not recorded).  CCS_EINVAL if that
- * iteration was not recorded. */
+/* Phase times of one iteration of the last CCS_K_PERSISTENT launch made while
+ * profiling (device timer between barriers): phase_us[0] score phase, [1]
+ * residual phase, [2..4] CTA 0's score sub-phases (fingerprints in, stream,
+ * queued candidates; -1 when not recorded).  CCS_EINVAL if that iteration was
+ * not recorded: launches of asynchronous calls, graphs and servers, and of a
+ * batch that needs several, are not. */
 CCS_API int ccs_profile_phases(int32_t iteration, double *phase_us);
 /* Number of kernels this library has launched since it was loaded. */
 CCS_API int64_t ccs_launch_count(void);

@@ -236,18 +236,8 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
             for (int u = 0; u < sizes[g]; ++u, ++t) sub[t].ctrl = header_ctrl(hdr, u);
         return autotune_groups(sub, sizes, groups, p, hdr, s, tuned);
     }
-    ccs_result *res =
-        dev_out ? dev_out : reinterpret_cast<ccs_result *>(rhdr + sizeof(EngineSync));
-    if ((rc = engine_run_batch(sub.data(), sizes, groups, count, p, kGroupIters, hdr, rhdr, s, res,
-                               capture)))
-        return rc;
-    if (dev_out) return CCS_OK;
-    rc = engine_results(rhdr, count, out, s);
-    if (rc == CCS_ETIMEOUT) {
-        const int rc2 = engine_stopped_results(sub.data(), count, hdr, out);
-        if (rc2) return rc2;
-    }
-    return rc;
+    return engine_run_batch(sub.data(), sizes, groups, count, p, kGroupIters, hdr, rhdr, s,
+                            dev_out, out, capture);
 }
 
 extern "C" int ccs_decode_batch(const ccs_problem *probs, int32_t count, const ccs_params *params,
@@ -293,6 +283,7 @@ extern "C" int ccs_batch_graph_create(const ccs_problem *probs, int32_t count,
 extern "C" int ccs_graph_launch(ccs_graph *g, ccs_stream_t stream) {
     if (!g || !g->exec) return CCS_EINVAL;
     count_launches(1);
+    prof_forget_stamps();
     CCS_CUDA_TRY(cudaGraphLaunch(g->exec, reinterpret_cast<cudaStream_t>(stream)));
     return CCS_OK;
 }

@@ -12,6 +12,13 @@
 
 namespace ccs {
 
+// Device timer, ns.
+__device__ __forceinline__ unsigned long long globaltimer() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // 8-bit fingerprint of a residual entry: 0 exactly when the value is zero
 // (+0.0 or -0.0), otherwise a hash of its bits in 1..255.  Equal values have
 // equal fingerprints, so a fingerprint count bounds the count of any value.

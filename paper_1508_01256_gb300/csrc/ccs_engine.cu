@@ -315,6 +315,32 @@ bool engine_fp_fits(const ProblemDev &pd, const ccs_params &prm) {
     return need <= smem_limit - fixed - 2 * stage_bytes;
 }
 
+// The stamps of a finished launch of `iterations` iterations to the profile.
+static int keep_stamps(const unsigned long long *stamps, int iterations, cudaStream_t s) {
+    std::vector<unsigned long long> h(kSubBase + 3 * kMaxStampIters);
+    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), stamps, sizeof(unsigned long long) * h.size(),
+                                 cudaMemcpyDeviceToHost, s));
+    CCS_CUDA_TRY(cudaStreamSynchronize(s));
+    prof_keep_stamps(h.data(), (int)h.size(), kSubBase);
+    for (int g = 0; g < iterations && 2 + 2 * g < (int)h.size(); ++g) {
+        const unsigned long long t0 = h[2 * g], t1 = h[1 + 2 * g], t2 = h[2 + 2 * g];
+        if (t1 >= t0 && t2 >= t1 && t0) {
+            prof_add(CCS_K_SCORE, (t1 - t0) * 1e-6);
+            prof_add(CCS_K_RESIDUAL, (t2 - t1) * 1e-6);
+            // CTA 0's view of the score phase: fingerprints in, stream done,
+            // queue done (0 when it had nothing to score)
+            const unsigned long long f = h[kSubBase + 3 * g], st = h[kSubBase + 3 * g + 1],
+                                     q = h[kSubBase + 3 * g + 2];
+            if (f >= t0 && st >= f && q >= st && q <= t1) {
+                prof_add(CCS_K_PHASE_FP, (f - t0) * 1e-6);
+                prof_add(CCS_K_PHASE_STREAM, (st - f) * 1e-6);
+                prof_add(CCS_K_PHASE_QUEUE, (q - st) * 1e-6);
+            }
+        }
+    }
+    return CCS_OK;
+}
+
 static void result_of(const DecodeCtrl &c, bool timed_out, ccs_result &out) {
     out.status = c.status;
     out.iterations = c.iteration;
@@ -338,7 +364,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     char *e = ws + sync_bytes(P);
     unsigned long long *stamps = reinterpret_cast<unsigned long long *>(e);
     e += stamps_bytes();
-    a.stamps = (profiling() && !dev_out && !small) ? stamps : nullptr;
+    a.stamps = (profiling() && !dev_out) ? stamps : nullptr;
     a.dev_out = dev_out;
     if (a.stamps) CCS_CUDA_TRY(cudaMemsetAsync(stamps, 0, stamps_bytes(), s));
 
@@ -357,9 +383,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
     }
 
     if (small) {
-        if ((rc = small_launch(pds, nullptr, 1, prm, a.sync, dev_out, s,
-                               true)))
-            return rc;
+        if ((rc = small_launch(pds, nullptr, 1, prm, a.sync, dev_out, a.stamps, s, true))) return rc;
     } else {
         void *args[] = {&a};
         const int ev = prof_start(CCS_K_PERSISTENT, s);
@@ -381,12 +405,6 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
         hdr = hdr_big.data();
     }
     CCS_CUDA_TRY(cudaMemcpyAsync(hdr, ws, hdr_bytes, cudaMemcpyDeviceToHost, s));
-    std::vector<unsigned long long> hst;
-    if (a.stamps) {
-        hst.resize(kSubBase + 3 * kMaxStampIters);
-        CCS_CUDA_TRY(cudaMemcpyAsync(hst.data(), stamps, sizeof(unsigned long long) * hst.size(),
-                                     cudaMemcpyDeviceToHost, s));
-    }
     CCS_CUDA_TRY(cudaStreamSynchronize(s));
     EngineSync hs;
     std::memcpy(&hs, hdr, sizeof(hs));
@@ -398,26 +416,7 @@ int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, c
         result_of(hc, herr != 0, out[p]);
         max_it = std::max(max_it, hc.iteration);
     }
-    if (a.stamps) prof_keep_stamps(hst.data(), (int)hst.size(), kSubBase);
-    if (a.stamps && !herr) {
-        // barrier 0 ends init; iteration g: score ends at 1+2g, residual at 2+2g
-        for (int g = 0; g < max_it && 2 + 2 * g < (int)hst.size(); ++g) {
-            const unsigned long long t0 = hst[2 * g], t1 = hst[1 + 2 * g], t2 = hst[2 + 2 * g];
-            if (t1 >= t0 && t2 >= t1 && t0) {
-                prof_add(CCS_K_SCORE, (t1 - t0) * 1e-6);
-                prof_add(CCS_K_RESIDUAL, (t2 - t1) * 1e-6);
-                // CTA 0's view of the score phase: fingerprints in, stream
-                // done, queue done (0 when it had nothing to score)
-                const unsigned long long f = hst[kSubBase + 3 * g], st = hst[kSubBase + 3 * g + 1],
-                                         q = hst[kSubBase + 3 * g + 2];
-                if (f >= t0 && st >= f && q >= st && q <= t1) {
-                    prof_add(CCS_K_PHASE_FP, (f - t0) * 1e-6);
-                    prof_add(CCS_K_PHASE_STREAM, (st - f) * 1e-6);
-                    prof_add(CCS_K_PHASE_QUEUE, (q - st) * 1e-6);
-                }
-            }
-        }
-    }
+    if (a.stamps && (rc = keep_stamps(stamps, herr ? 0 : max_it, s))) return rc;
     if (herr) {
         set_last_error("a bounded device wait exceeded the watchdog (%d ms)",
                        prm.watchdog_ms > 0 ? prm.watchdog_ms : 2000);
@@ -435,6 +434,33 @@ size_t engine_resume_header_bytes(int P) {
     return resume_results_bytes(P) + stamps_bytes() + align_up(sizeof(ProblemDev) * (size_t)P, 256);
 }
 
+// The result area of a header (P entries) to the host.  Waits for `s`.
+static int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s) {
+    const size_t bytes = sizeof(EngineSync) + sizeof(ccs_result) * (size_t)P;
+    std::vector<char> h(bytes);
+    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), rhdr, bytes, cudaMemcpyDeviceToHost, s));
+    CCS_CUDA_TRY(cudaStreamSynchronize(s));
+    EngineSync hs;
+    std::memcpy(&hs, h.data(), sizeof(hs));
+    std::memcpy(out, h.data() + sizeof(EngineSync), sizeof(ccs_result) * (size_t)P);
+    if (hs.error) {
+        for (int p = 0; p < P; ++p) out[p].error = CCS_ETIMEOUT;
+        set_last_error("a bounded device wait exceeded the watchdog");
+        return CCS_ETIMEOUT;
+    }
+    return CCS_OK;
+}
+
+// Results of a batch whose launch timed out before it wrote them: each
+// problem as its control block stands.
+static int engine_stopped_results(const ProblemDev *pds, int P, char *hdr, ccs_result *out) {
+    std::vector<DecodeCtrl> c(P);
+    CCS_CUDA_TRY(cudaMemcpy(c.data(), header_ctrl(hdr, 0), sizeof(DecodeCtrl) * (size_t)P,
+                            cudaMemcpyDeviceToHost));
+    for (int t = 0; t < P; ++t) result_of(c[t], true, out[pds[t].out_slot]);
+    return CCS_OK;
+}
+
 // A batch.  pds: the `rest` = sum of sizes[0..groups) problems of the launch
 // classes back to back, then the count - rest that go out as one launch of
 // the small engine; their out_slot the caller's index, their control blocks
@@ -447,11 +473,15 @@ size_t engine_resume_header_bytes(int P) {
 // over all of them resumes the ones still running, so the tails share
 // iterations.
 //
-// Results go to res[out_slot].  Enqueued on `s`, or, with `capture`, made a
+// Results go to dev_out[out_slot]: enqueued on `s`, or, with `capture`, made a
 // CUDA graph that replays the launches (the descriptors are uploaded now).
+// Without dev_out the batch is run to its end and they go to out[out_slot];
+// the phases of a batch that is one launch are then kept while profiling.
 int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
                      const ccs_params &prm, int group_iters, char *hdr, char *rhdr,
-                     cudaStream_t s, ccs_result *res, cudaGraphExec_t *capture) {
+                     cudaStream_t s, ccs_result *dev_out, ccs_result *out,
+                     cudaGraphExec_t *capture) {
+    ccs_result *res = dev_out ? dev_out : reinterpret_cast<ccs_result *>(rhdr + sizeof(EngineSync));
     int rest = 0;
     for (int g = 0; g < groups; ++g) rest += sizes[g];
     ProblemDev *d_fresh = reinterpret_cast<ProblemDev *>(hdr + sync_bytes(count) + stamps_bytes());
@@ -459,6 +489,11 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
         reinterpret_cast<ProblemDev *>(rhdr + resume_results_bytes(count) + stamps_bytes());
     EngineSync *sync = reinterpret_cast<EngineSync *>(rhdr);
     const int launches = groups > 1 ? groups + 1 : groups;
+    unsigned long long *stamps = nullptr;
+    if (profiling() && !dev_out && !capture && launches <= 1) {
+        stamps = reinterpret_cast<unsigned long long *>(hdr + sync_bytes(count));
+        CCS_CUDA_TRY(cudaMemsetAsync(stamps, 0, stamps_bytes(), s));
+    }
     std::vector<ProblemDev> fresh(pds, pds + count), again(pds, pds + count);
     for (int t = 0; t < count; ++t) {
         fresh[t].flags |= kPdFresh;
@@ -476,6 +511,7 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
         fill_args(a, plans[l], P, prm);
         a.sync = sync;
         a.dev_out = last ? res : nullptr;
+        a.stamps = stamps;
         if (rest == 1) {
             a.single = *host;  // a lone problem
         } else {
@@ -504,7 +540,7 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
         int rc;
         if (rest < count &&
             (rc = small_launch(pds + rest, count > 1 ? d_fresh + rest : nullptr, count - rest, prm,
-                               sync, res, cs, !capture)))
+                               sync, res, launches ? nullptr : stamps, cs, !capture)))
             return rc;
         for (int l = 0; l < launches; ++l) {
             const LaunchPlan &L = plans[l];
@@ -521,7 +557,24 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
         }
         return CCS_OK;
     };
-    if (!capture) return enqueue(s);
+    if (!capture) {
+        int rc = enqueue(s);
+        if (rc || dev_out) return rc;
+        rc = engine_results(rhdr, count, out, s);
+        if (rc == CCS_ETIMEOUT) {
+            const int rc2 = engine_stopped_results(pds, count, hdr, out);
+            if (rc2) return rc2;
+        }
+        if (!rc && stamps) {
+            // the engine's iterations are the longest decode's; on chip the
+            // first (largest) problem's are stamped
+            int iterations = 0;
+            for (int t = 0; t < (launches ? rest : 1); ++t)
+                iterations = std::max(iterations, out[pds[t].out_slot].iterations);
+            rc = keep_stamps(stamps, iterations, s);
+        }
+        return rc;
+    }
     cudaStream_t cs;
     CCS_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
@@ -536,33 +589,6 @@ int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
     cudaStreamDestroy(cs);
     if (rc) return rc;
     if (e != cudaSuccess) return cuda_fail(e, "capturing the batch");
-    return CCS_OK;
-}
-
-// The result area of a header (P entries) to the host.  Waits for `s`.
-int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s) {
-    const size_t bytes = sizeof(EngineSync) + sizeof(ccs_result) * (size_t)P;
-    std::vector<char> h(bytes);
-    CCS_CUDA_TRY(cudaMemcpyAsync(h.data(), rhdr, bytes, cudaMemcpyDeviceToHost, s));
-    CCS_CUDA_TRY(cudaStreamSynchronize(s));
-    EngineSync hs;
-    std::memcpy(&hs, h.data(), sizeof(hs));
-    std::memcpy(out, h.data() + sizeof(EngineSync), sizeof(ccs_result) * (size_t)P);
-    if (hs.error) {
-        for (int p = 0; p < P; ++p) out[p].error = CCS_ETIMEOUT;
-        set_last_error("a bounded device wait exceeded the watchdog");
-        return CCS_ETIMEOUT;
-    }
-    return CCS_OK;
-}
-
-// Results of a batch whose launch timed out before it wrote them: each
-// problem as its control block stands.
-int engine_stopped_results(const ProblemDev *pds, int P, char *hdr, ccs_result *out) {
-    std::vector<DecodeCtrl> c(P);
-    CCS_CUDA_TRY(cudaMemcpy(c.data(), header_ctrl(hdr, 0), sizeof(DecodeCtrl) * (size_t)P,
-                            cudaMemcpyDeviceToHost));
-    for (int t = 0; t < P; ++t) result_of(c[t], true, out[pds[t].out_slot]);
     return CCS_OK;
 }
 

@@ -45,7 +45,6 @@ namespace ccs {
 constexpr int kTile = 32;
 constexpr int kMaxBlocks = 1024;
 constexpr int kMaxProblems = 4096;  // per launch: their status and weight prefix live on chip
-constexpr int kMaxStampIters = 1024;
 constexpr int kMaxStages = 6;
 constexpr int kOvfCap = 512;       // overflow rows listed per CTA and segment
 constexpr int kQueueCap = 2048;     // most candidate columns queued per CTA and segment
@@ -62,7 +61,6 @@ constexpr int kWbufPerWarp = 32;    // buffered candidate columns per consumer w
 // memory only.
 template <int DMAX>
 constexpr int kWbufEntry = 1 + (DMAX + 1) / 2;
-constexpr int kSubBase = 3 * kMaxStampIters + 2;  // CTA-0 score sub-phase stamps start here
 constexpr int kRowDrivenDiv = 64;   // row-driven score phase while ||r||_0 <= m / kRowDrivenDiv
 constexpr long long kRowDrivenMinEntries = 64ll << 20;  // ... and the CSC (n d entries) streams
                                                        // from HBM, not from L2
@@ -92,12 +90,6 @@ struct EngineArgs {
 };
 
 // ---- device helpers --------------------------------------------------------
-
-__device__ __forceinline__ unsigned long long globaltimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;

@@ -16,6 +16,12 @@ constexpr int kSlotRec = 16;        // ints per row record: count, then kSlots c
 constexpr int kMaxSortRow = 32768;  // longest CSR row sorted on chip
 constexpr int kRunning = -1;        // DecodeCtrl::status while iterating
 
+// Phase stamps of a profiled launch (device timer, ns): [0] init done, [1 + 2 g]
+// score phase of iteration g done, [2 + 2 g] its residual; from kSubBase on,
+// three an iteration: fingerprints in, columns tested, candidates scored.
+constexpr int kMaxStampIters = 1024;
+constexpr int kSubBase = 3 * kMaxStampIters + 2;
+
 // Bits of ccs_params.debug_flags that both engines know (the others are in
 // ccs_engine_kernel.cuh).
 constexpr int kFlagOrdered = 2;     // test hook: ordered residual from the start
@@ -179,6 +185,7 @@ void prof_stop(int slot, cudaStream_t s);
 void prof_collect();
 void prof_add(int kind, double ms);
 void prof_keep_stamps(const unsigned long long *st, int count, int sub_base);
+void prof_forget_stamps();
 
 // host-driven loop (ccs_decode.cu)
 int decode_host_loop(const ProblemDev &P, const ccs_params &p, ccs_result *out, cudaStream_t s);
@@ -212,7 +219,7 @@ size_t max_dynamic_smem(int dev, const void *fn);
 // (alone: nothing else shares the GPU with it).
 bool small_route(const ProblemDev &pd, const ccs_params &prm, bool alone);
 int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_params &prm,
-                 EngineSync *sync, ccs_result *dev_out,
+                 EngineSync *sync, ccs_result *dev_out, unsigned long long *stamps,
                  cudaStream_t s, bool timed);
 
 // The expander's construction (ccs_setup.cu): all of it enqueued, then what
@@ -226,13 +233,12 @@ int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc
 
 int engine_resume(ProblemDev *pds, int P, const ccs_params &prm, int iter_budget, ccs_result *out,
                   char *hdr, cudaStream_t s);
-// A batch (see ccs_engine.cu), run now or captured in a CUDA graph, and the
-// read-back of a header's results.
+// A batch (see ccs_engine.cu): enqueued with its results going to dev_out, or
+// captured in a CUDA graph, or (dev_out null) run to its end, results to out.
 int engine_run_batch(ProblemDev *pds, const int *sizes, int groups, int count,
                      const ccs_params &prm, int group_iters, char *hdr, char *rhdr,
-                     cudaStream_t s, ccs_result *res, cudaGraphExec_t *capture);
-int engine_results(char *rhdr, int P, ccs_result *out, cudaStream_t s);
-int engine_stopped_results(const ProblemDev *pds, int P, char *hdr, ccs_result *out);
+                     cudaStream_t s, ccs_result *dev_out, ccs_result *out,
+                     cudaGraphExec_t *capture);
 int check_params(const ccs_params *p, int d);
 
 }  // namespace ccs

@@ -40,6 +40,7 @@ bool profiling() { return g_on; }
 int prof_start(int kind, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g_mu);
     if (!g_on) return -1;
+    if (kind == CCS_K_PERSISTENT) g_stamps.clear();  // those of an earlier launch
     Pending p{kind, take_event(), take_event()};
     if (!p.start || !p.stop) return -1;
     cudaEventRecord(p.start, s);
@@ -74,6 +75,11 @@ void prof_keep_stamps(const unsigned long long *st, int count, int sub_base) {
     std::lock_guard<std::mutex> lk(g_mu);
     g_stamps.assign(st, st + count);
     g_sub_base = sub_base;
+}
+
+void prof_forget_stamps() {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (g_on) g_stamps.clear();
 }
 
 void prof_add(int kind, double ms) {

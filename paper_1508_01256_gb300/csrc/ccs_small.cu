@@ -68,6 +68,7 @@ struct SmallArgs {
     int alpha, mode, max_iter, debug_flags, shifted;
     EngineSync *sync;
     ccs_result *dev_out;       // or null
+    unsigned long long *stamps;  // phases of the first problem (or null)
 };
 
 // Updates of another CTA's shared memory: `local` is the place in this CTA's,
@@ -296,6 +297,11 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
     };
     if (tid == 0 && s.status == kRunning) next_form();
     cl.sync();  // every CTA's copy is ready for the others' updates
+    auto stamp = [&](int at) {
+        if (a.stamps && tid == 0 && rank == 0 && s.problem == 0 && s.it < kMaxStampIters)
+            a.stamps[at] = globaltimer();
+    };
+    stamp(0);
 
     while (s.status == kRunning) {
         const int it = s.it, par = it & 1;
@@ -318,6 +324,8 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
                 }
             }
         }
+
+        stamp(kSubBase + 3 * it);
 
         // ---- score: the columns the fingerprints let through are queued, ----
         // then scored exactly on full warps
@@ -345,6 +353,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
             }
         }
         __syncthreads();
+        stamp(kSubBase + 3 * it + 1);
         unsigned long long xnew = 0;
         for (int e = tid; e < s.queued; e += kSmallThreads) {
             const int j = S.queue[e];
@@ -396,12 +405,14 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
         xnew = warp_max_bits(xnew);
         if (lane == 0 && xnew) atomicMax(&s.xnew, xnew);
         __syncthreads();
+        stamp(kSubBase + 3 * it + 2);
         if (tid < C) {
             cluster_set(cluster_addr(&s.all_acc[par][rank], tid), s.acc);
             cluster_set(cluster_addr(&s.all_xnew[par][rank], tid), s.xnew);
         }
         if (tid == 0) s.rmax = 0;
         cl.sync();
+        stamp(1 + 2 * it);
 
         // ---- the other CTAs' accepted columns into this copy --------------
         const unsigned mine = lane < C ? s.all_acc[par][lane] : 0u;
@@ -512,6 +523,7 @@ __device__ __forceinline__ void small_decode(const SmallArgs &a, const ProblemDe
         }
         __syncthreads();
 
+        stamp(2 + 2 * it);
         // ---- stop rule, as in the engine --------------------------------
         if (tid == 0) {
             const bool empty = total == 0;
@@ -636,10 +648,10 @@ static int small_clusters(int dev, int C) {
 
 // P problems (descriptors `pds` on the host; `dev` the same ones in device
 // memory, or null for a single one), enqueued on `s` (`timed`: with the
-// profiler's events, which a capture leaves out).  The sync word's
-// `next` starts at zero.
+// profiler's events, which a capture leaves out; `stamps`, or null: the phases
+// of the first).  The sync word's `next` starts at zero.
 int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_params &prm,
-                 EngineSync *sync, ccs_result *dev_out,
+                 EngineSync *sync, ccs_result *dev_out, unsigned long long *stamps,
                  cudaStream_t s, bool timed) {
     long long entries = 0;
     for (int p = 0; p < P; ++p) {
@@ -670,6 +682,7 @@ int small_launch(const ProblemDev *pds, const ProblemDev *dev, int P, const ccs_
     a.shifted = prm.shifted;
     a.sync = sync;
     a.dev_out = dev_out;
+    a.stamps = stamps;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
     cfg.gridDim = dim3((unsigned)(C * (P < most ? P : most)));
