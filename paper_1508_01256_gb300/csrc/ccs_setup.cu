@@ -175,19 +175,49 @@ k_scan_local(int m, const int32_t *deg, int64_t *ptr, int64_t *sums, int *max_de
     if (threadIdx.x == kScanBlock - 1) sums[blockIdx.x] = inc;
 }
 
-// ptr += the totals of the blocks before (each block sums them itself).
-__global__ void __launch_bounds__(kScanBlock) k_scan_add(int m, int64_t *ptr, const int64_t *sums) {
+// ptr += the totals of the blocks before.  Up to kScanBlock blocks (m = 2^20)
+// each sums them itself, one load a thread; beyond, k_scan_totals has turned
+// them into prefixes (`scanned`): the sums would be quadratic in m (33 ms
+// more at m = 2^29, 1.8 ms at 2^27).
+__global__ void __launch_bounds__(kScanBlock)
+k_scan_add(int m, int64_t *ptr, const int64_t *sums, bool scanned) {
     __shared__ unsigned long long before;
     const int i = blockIdx.x * kScanBlock + threadIdx.x;
-    if (threadIdx.x == 0) before = 0;
+    if (threadIdx.x == 0) before = scanned ? (unsigned long long)sums[blockIdx.x] : 0;
     __syncthreads();
-    long long v = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanBlock) v += sums[b];
-    v = warp_sum_ll(v);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&before, (unsigned long long)v);
-    __syncthreads();
+    if (!scanned) {
+        const long long v = warp_sum_ll(threadIdx.x < blockIdx.x ? sums[threadIdx.x] : 0);
+        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&before, (unsigned long long)v);
+        __syncthreads();
+    }
     if (i == 0) ptr[0] = 0;
     if (i < m) ptr[i + 1] += (long long)before;
+}
+
+// Exclusive prefix of the block totals, in place (one block, a run of
+// consecutive totals a thread).
+__global__ void __launch_bounds__(kScanBlock) k_scan_totals(int nblocks, int64_t *sums) {
+    __shared__ long long warp_tot[kScanBlock / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (nblocks + kScanBlock - 1) / kScanBlock;
+    const int b0 = min(nblocks, (int)threadIdx.x * per), b1 = min(nblocks, b0 + per);
+    long long sum = 0;
+    for (int b = b0; b < b1; ++b) sum += sums[b];
+    long long inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    long long run = inc - sum;
+    for (int w = 0; w < warp; ++w) run += warp_tot[w];
+    for (int b = b0; b < b1; ++b) {
+        const long long v = sums[b];
+        sums[b] = run;
+        run += v;
+    }
 }
 
 // Entries of a k_generate_columns that packed their ranks: each goes to its
@@ -1079,7 +1109,9 @@ static int expander_build(int32_t n, int32_t m, uint64_t seed, int32_t *csc_rows
     k_generate_columns<D><<<(n + kGenBlock - 1) / kGenBlock, kGenBlock, 0, s>>>(
         n, m, seed, pl.rank_shift, csc_rows, w.deg);
     k_scan_local<<<w.nblocks, kScanBlock, 0, s>>>(m, w.deg, csr_ptr, w.sums, w.max_deg);
-    k_scan_add<<<w.nblocks, kScanBlock, 0, s>>>(m, csr_ptr, w.sums);
+    const bool scanned = w.nblocks > kScanBlock;
+    if (scanned) k_scan_totals<<<1, kScanBlock, 0, s>>>(w.nblocks, w.sums);
+    k_scan_add<<<w.nblocks, kScanBlock, 0, s>>>(m, csr_ptr, w.sums, scanned);
     CCS_CUDA_TRY(cudaGetLastError());
     if (pl.rank_shift) {
         k_place_ranked<D><<<grid_for((edges + 3) / 4, 256), 256, 0, s>>>(

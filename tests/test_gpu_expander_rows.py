@@ -1,0 +1,61 @@
+"""Expanders of very many rows: the row offsets on both sides of the sizes at
+which the block totals get a scan of their own (1024 blocks of 1024 rows), and
+a construction time that grows with the number of rows, not its square."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ccs():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1508_01256_gb300 import build, ccs
+    build.build()
+    return ccs
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+    oracle.build()
+    return oracle
+
+
+# n > 2^25: six bits left for a row beside a column, so that these m take the
+# row-by-row construction
+@pytest.mark.parametrize("m", [2 ** 20 - 1, 2 ** 20, 2 ** 20 + 1, 2 ** 21 + 1025, 3 * 2 ** 20])
+def test_offsets_around_the_scan_of_totals(ccs, orc, m):
+    n, d = 2 ** 25 + 1, 1
+    csc, ptr, cols = ccs.make_expander(n, m, d, 9 + m)
+    A = orc.make_expander(n, m, d, 9 + m)
+    ptr_ref, cols_ref = orc.transpose(A, m)
+    assert np.array_equal(csc.cpu().numpy(), A)
+    assert np.array_equal(ptr.cpu().numpy(), ptr_ref)
+    assert np.array_equal(cols.cpu().numpy(), cols_ref)
+
+
+def test_time_grows_with_the_rows(ccs):
+    """Four times the rows: about four times the passes over them (a sum over
+    all totals before it in every block makes it 13 times)."""
+    import torch
+
+    def best(m):
+        n, d = 1003, 3
+        csc = torch.empty(n, d, dtype=torch.int32, device="cuda")
+        ptr = torch.empty(m + 1, dtype=torch.int64, device="cuda")
+        cols = torch.empty(n * d, dtype=torch.int32, device="cuda")
+        ws = ccs.workspace(ccs.ccs_workspace_size(ccs.OP_MAKE_EXPANDER, n, m, d))
+        times = []
+        for _ in range(4):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            ccs.ccs_make_expander(n, m, d, 77, csc, ptr, cols, ws)
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        return min(times)
+
+    assert best(2 ** 29) < 8 * best(2 ** 27)
