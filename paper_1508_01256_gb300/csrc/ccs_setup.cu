@@ -183,40 +183,50 @@ __global__ void __launch_bounds__(kScanBlock)
 k_scan_add(int m, int64_t *ptr, const int64_t *sums, bool scanned) {
     __shared__ unsigned long long before;
     const int i = blockIdx.x * kScanBlock + threadIdx.x;
-    if (threadIdx.x == 0) before = scanned ? (unsigned long long)sums[blockIdx.x] : 0;
-    __syncthreads();
-    if (!scanned) {
-        const long long v = warp_sum_ll(threadIdx.x < blockIdx.x ? sums[threadIdx.x] : 0);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&before, (unsigned long long)v);
-        __syncthreads();
-    }
     if (i == 0) ptr[0] = 0;
+    if (scanned) {
+        if (i < m) ptr[i + 1] += sums[blockIdx.x];
+        return;
+    }
+    if (threadIdx.x == 0) before = 0;
+    __syncthreads();
+    const long long v = warp_sum_ll(threadIdx.x < blockIdx.x ? sums[threadIdx.x] : 0);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&before, (unsigned long long)v);
+    __syncthreads();
     if (i < m) ptr[i + 1] += (long long)before;
 }
 
-// Exclusive prefix of the block totals, in place (one block, a run of
-// consecutive totals a thread).
+// Exclusive prefix of the block totals, in place: one block, each warp a
+// stretch of them, 32 consecutive ones at a time.
 __global__ void __launch_bounds__(kScanBlock) k_scan_totals(int nblocks, int64_t *sums) {
+    constexpr int kU = 8;  // loads in flight
     __shared__ long long warp_tot[kScanBlock / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per = (nblocks + kScanBlock - 1) / kScanBlock;
-    const int b0 = min(nblocks, (int)threadIdx.x * per), b1 = min(nblocks, b0 + per);
+    const int per = (nblocks + kScanBlock - 1) / kScanBlock * 32;
+    const int b0 = min(nblocks, warp * per), b1 = min(nblocks, b0 + per);
     long long sum = 0;
-    for (int b = b0; b < b1; ++b) sum += sums[b];
-    long long inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) warp_tot[warp] = inc;
+#pragma unroll kU
+    for (int b = b0 + lane; b < b1; b += 32) sum += sums[b];
+    sum = warp_sum_ll(sum);
+    if (lane == 0) warp_tot[warp] = sum;
     __syncthreads();
-    long long run = inc - sum;
+    long long run = 0;
     for (int w = 0; w < warp; ++w) run += warp_tot[w];
-    for (int b = b0; b < b1; ++b) {
-        const long long v = sums[b];
-        sums[b] = run;
-        run += v;
+    for (int b = b0 + lane; b - lane < b1; b += 32 * kU) {
+        long long v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) v[u] = b + 32 * u < b1 ? sums[b + 32 * u] : 0;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            long long inc = v[u];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            if (b + 32 * u < b1) sums[b + 32 * u] = run + inc - v[u];
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        }
     }
 }
 
