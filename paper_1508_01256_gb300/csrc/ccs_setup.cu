@@ -124,6 +124,11 @@ k_generate_columns(int n, int m, uint64_t seed, int shift, int32_t *csc_rows, in
 
 constexpr int kScanBlock = 1024;
 constexpr int kWarpSortCap = 512;   // longest row a warp sorts in registers
+// From here on the rows' counters and offsets leave L2, and entries carry their
+// ranks from the count to the placing instead of counting again (n = 2^25 + 1:
+// m = 2^24, d = 7 18.7 ms against 23.7; m = 2^22, d = 5 10.7 against 10.4; m =
+// 2^20, d = 3 5.8 against 4.2).
+constexpr int kRankedRows = 1 << 22;
 constexpr int kGroupEntries = 36864;  // entries a group of rows has at most, on average
 constexpr int kMaxGroups = 8192;      // counted on chip
 constexpr int kMaxGroupRowBits = 12;
@@ -964,8 +969,6 @@ struct ExpanderPlan {
     size_t draw_smem, deal_smem, sort_smem;
     // otherwise:
     int rank_shift;         // > 0: ranks ride above this bit of the row indices
-    int cap;                // row length the sort is sized for
-    bool sort_early;        // sorted before the longest row is known
 };
 
 // Entries that a row (or a group of rows) with `mean` of them on average is
@@ -987,15 +990,9 @@ static int expander_plan(int32_t n, int32_t m, int32_t d, ExpanderPlan &pl) {
     CCS_CUDA_TRY(cudaGetDevice(&dev));
     CCS_CUDA_TRY(cudaDeviceGetAttribute(&pl.sms, cudaDevAttrMultiProcessorCount, dev));
     CCS_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    pl.cap = likely_most(mean, edges);
-    if (pl.cap > kMaxSortRow) pl.cap = kMaxSortRow;
-    // Rows that most likely hold one column at most (fewer than one pair of
-    // entries in a row on average) need no sort, and passing over them for
-    // one takes longer than all the rest (n = 1003, m = 2^29, d = 3: 33 ms
-    // instead of 6.8).
-    pl.sort_early = (double)edges * edges >= 2.0 * m;
     const int row_bits = m > 1 ? bits_for(m) : 1;
-    pl.rank_shift = ((long long)pl.cap >> (32 - row_bits)) == 0 ? row_bits : 0;
+    const long long likely = std::min(likely_most(mean, edges), kMaxSortRow);
+    pl.rank_shift = m > kRankedRows && (likely >> (32 - row_bits)) == 0 ? row_bits : 0;
 
     // groups of up to kGroupEntries entries, and enough of them for every SM
     pl.groups = 0;
@@ -1138,7 +1135,7 @@ static int expander_build(int32_t n, int32_t m, uint64_t seed, int32_t *csc_rows
                                                             csr_cols);
     }
     CCS_CUDA_TRY(cudaGetLastError());
-    return pl.sort_early ? sort_rows(n, m, pl.cap, csr_ptr, csr_cols, s) : CCS_OK;
+    return CCS_OK;  // the rows are sorted once the longest one is known
 }
 
 typedef int (*build_fn)(int32_t, int32_t, uint64_t, int32_t *, int64_t *, int32_t *,
@@ -1152,9 +1149,9 @@ static build_fn expander_builder(int d) {
     return fns[d - 1];
 }
 
-// The expander's whole construction, enqueued on `s` and sized for the row
-// lengths a uniform draw has.  *max_deg_dev receives the device address of
-// the largest row degree, which expander_finish needs on the host.
+// The expander's construction up to the sort of single rows, enqueued on `s`.
+// *max_deg_dev receives the device address of the largest row degree, which
+// expander_finish needs on the host.
 // Arguments already checked.
 int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
                          int64_t *csr_ptr, int32_t *csr_cols, void *ws, cudaStream_t s,
@@ -1167,9 +1164,13 @@ int expander_build_async(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t
     return expander_builder(d)(n, m, seed, csc_rows, csr_ptr, csr_cols, w, pl, s);
 }
 
-// What is left once the largest row degree is known: nothing, as a rule.
-// CCS_EINVAL when a row is longer than the on-chip sort takes.  Enqueued on
-// `s`; *again: whether anything was.
+// What is left once the largest row degree is known: nothing after a grouped
+// construction, as a rule; else the sort of the rows, sized by the longest
+// one (sizing it beforehand by what rows are unlikely to pass took up to twice
+// as long: n = 2^25 + 1, m = 2^20, d = 1 0.58 ms against 0.27; and where no
+// row holds two columns there is nothing to sort: n = 1003, m = 2^29, d = 3
+// 26 ms spared).  CCS_EINVAL when a row is longer than the on-chip sort
+// takes.  Enqueued on `s`; *again: whether anything was.
 int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc_rows,
                     int64_t *csr_ptr, int32_t *csr_cols, void *ws, int host_max, cudaStream_t s,
                     bool *again) {
@@ -1191,7 +1192,7 @@ int expander_finish(int32_t n, int32_t m, int32_t d, uint64_t seed, int32_t *csc
                        kMaxSortRow);
         return CCS_EINVAL;
     }
-    if (pl.groups || host_max <= (pl.sort_early ? pl.cap : 1)) return CCS_OK;
+    if (pl.groups || host_max <= 1) return CCS_OK;
     *again = true;
     if (pl.rank_shift && ((long long)host_max >> (32 - pl.rank_shift)) != 0) {
         // ranks that did not fit their bits: draw again without them

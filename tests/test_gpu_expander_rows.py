@@ -38,6 +38,18 @@ def test_offsets_around_the_scan_of_totals(ccs, orc, m):
     assert np.array_equal(cols.cpu().numpy(), cols_ref)
 
 
+@pytest.mark.parametrize("m", [2 ** 22, 2 ** 22 + 1])
+def test_both_ways_to_place_the_entries(ccs, orc, m):
+    """Counted again, and by the ranks that the count handed out."""
+    n, d = 2 ** 24 + 3, 3
+    csc, ptr, cols = ccs.make_expander(n, m, d, 5)
+    A = orc.make_expander(n, m, d, 5)
+    ptr_ref, cols_ref = orc.transpose(A, m)
+    assert np.array_equal(csc.cpu().numpy(), A)
+    assert np.array_equal(ptr.cpu().numpy(), ptr_ref)
+    assert np.array_equal(cols.cpu().numpy(), cols_ref)
+
+
 def test_time_grows_with_the_rows(ccs):
     """Four times the rows: about four times the passes over them (a sum over
     all totals before it in every block makes it 13 times)."""
