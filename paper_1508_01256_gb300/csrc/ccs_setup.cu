@@ -732,12 +732,34 @@ __device__ __forceinline__ double measured_value(const double *sc, const double 
 
 // Bit b of `bits`: columns [b 2^shift, (b + 1) 2^shift) hold a nonzero.  A
 // warp makes whole words: 32 columns at a time, coalesced.
+//
+// A dense x is not marked: every block looks at the same sample, eight
+// stretches of 32 columns spread over x, and when more than kMarkDense of
+// them hold a nonzero the word behind the bits says so and the rows gather
+// everything.  The sample decides the way only, never the result.  Marks pay
+// below ~2 % of nonzeros; beyond, the lines below hold gathering every entry a
+// warp a row, marks, and the unmarked rows here, in us:
+//   n = 2^20, m = 10486, d = 7:   1 % 50, 47, -;  5 % 59, 70, 65;  10 % 86, 96, 89
+//   n = 2^23, m = 2^16, d = 7:   10 % 511, 543, 522;  100 % 3726, 3803, 3781
+//   n = 2^24, m = 16777, d = 9:  10 % 1339, 1321, 1279;  100 % 9697, 9819, 9776
+// (the first has no second launch).  Tried: a dense x measured a warp a row by
+// the marking blocks, which the GPU holds all at once: 1545 us instead of 1279
+// in the last line, its rows being shared out less evenly.  A sample of 1024
+// single columns cost every x 3-6 us.
+constexpr int kMarkThreads = 256;
+constexpr int kMarkDense = 5;
 template <bool kScaled>
-__global__ void k_mark_nonzeros(int n, int shift, const double *sc, const double *x,
-                                unsigned *bits) {
+__global__ void __launch_bounds__(kMarkThreads)
+k_mark_nonzeros(int n, int shift, const double *sc, const double *x, unsigned *bits) {
     const int lane = threadIdx.x & 31;
     const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
     const long long words = (((long long)n - 1) >> shift) / 32 + 1;
+    const long long at =
+        (long long)__umulhi((threadIdx.x >> 5) * 0x9e3779b9u, (unsigned)n) + lane;
+    const bool dense = __syncthreads_count(at < n && measured_value<kScaled>(sc, x, at) != 0.0) >
+                       kMarkDense;
+    if (blockIdx.x == 0 && threadIdx.x == 0) bits[words] = dense;
+    if (dense) return;
     for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < words;
          w += warps) {
         const long long c0 = w << (shift + 5);
@@ -776,7 +798,8 @@ k_measure_marked(int m, int shift, int words, int batch, const int64_t *ptr, con
     extern __shared__ unsigned bits[];
     __shared__ int next;
     const unsigned *src = reinterpret_cast<const unsigned *>(y);
-    for (int w = threadIdx.x; w < words; w += kMarkBlock) bits[w] = __ldcg(src + w);
+    const bool dense = __ldcg(src + words) != 0;
+    for (int w = threadIdx.x; w < words; w += kMarkBlock) bits[w] = dense ? ~0u : __ldcg(src + w);
     const int lane = threadIdx.x & 31;
     const int r0 = (int)((long long)m * blockIdx.x / gridDim.x);
     const int r1 = (int)((long long)m * (blockIdx.x + 1) / gridDim.x);
@@ -1217,13 +1240,13 @@ static int measure_rows(int32_t n, int32_t m, int32_t d, const int64_t *csr_ptr,
         CCS_CUDA_TRY(cudaGetDevice(&dev));
         CCS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         CCS_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        // as many bits as y (64 m) and shared memory hold
-        const long long room = std::min(64ll * m, (long long)kMarkBytes * 8);
+        // as many bits as y (64 m, less a word) and shared memory hold
+        const long long room = std::min(64ll * m - 32, (long long)kMarkBytes * 8);
         int shift = 0;
         while (((((long long)n - 1) >> shift) / 32 + 1) * 32 > room) ++shift;
         const int words = (int)((((long long)n - 1) >> shift) / 32 + 1);
         if (coop && shift <= kMarkMaxShift) {
-            k_mark_nonzeros<kScaled><<<sms * 8, 256, 0, s>>>(n, shift, sc, x,
+            k_mark_nonzeros<kScaled><<<sms * 8, kMarkThreads, 0, s>>>(n, shift, sc, x,
                                                              reinterpret_cast<unsigned *>(y));
             CCS_CUDA_TRY(cudaGetLastError());
             const size_t smem = (size_t)words * 4;
