@@ -137,3 +137,25 @@ def test_clusters_that_start_at_different_times(ccs, orc):
                 (refs[q]["status"], refs[q]["iterations"], 0)
             assert np.array_equal(x.cpu().numpy(), refs[q]["x_hat"])
         graph.close()
+
+
+# n d just below and above a cluster size's entries; the last CTA's part short,
+# and empty (160 columns a part: 6 full ones, 70 columns, none)
+@pytest.mark.parametrize("shape, ctas", [((585, 70, 7, 7), 1), ((586, 70, 7, 7), 2), ((1170, 130, 7, 30), 2),
+                                         ((1171, 130, 7, 30), 4), ((2341, 300, 7, 30), 8),
+                                         ((1030, 160, 16, 12), 8)])
+def test_cluster_sizes(ccs, orc, shape, ctas):
+    n, m, d, k = shape
+    C, pitch = _parts(n, d)
+    assert C == ctas and (shape[0] != 1030 or 7 * pitch >= n)
+    for values in ("gauss-grid", "gauss-raw"):
+        p = inputs.make_problem(n, m, d, k, 300 + n, values)
+        items = device_problem(ccs, p)
+        A, y = oracle_problem(orc, p)
+        ref = orc.parallel_l0(A, m, y, max_iter=30)
+        for flags in (0, 2, 4):
+            g = ccs.decode_parallel_l0(*items, max_iter=30, debug_flags=flags)
+            assert_same_decode(g, ref)
+            h = ccs.decode_batch([items, items], max_iter=30, history=True, debug_flags=flags)
+            for b in h:
+                assert_same_decode(b, ref)
