@@ -89,7 +89,11 @@ enum {
                                   are decoded there (no grid barriers), the
                                   others, and a server's, by the persistent
                                   engine; schedule or debug_flags beyond
-                                  bits 1-2 keep to the persistent engine     */
+                                  bits 1-2 keep to the persistent engine.
+                                  On chip the only waits are the hardware
+                                  barriers of a cluster, whose CTAs are
+                                  resident together: watchdog_ms does not
+                                  bound them                                 */
     CCS_ENGINE_HOST_LOOP = 1,  /* one launch per phase, host checks the stop
                                   rule after every iteration                 */
     CCS_ENGINE_PERSISTENT = 3  /* one cooperative launch runs every
@@ -104,7 +108,8 @@ typedef struct {
     int32_t max_iter;     /* iteration cap, >= 0; default 100                 */
     int32_t score_mode;   /* CCS_SCORE_*; default CCS_SCORE_L0_DECREASE       */
     int32_t engine;       /* CCS_ENGINE_*; default CCS_ENGINE_AUTO            */
-    int32_t watchdog_ms;  /* bound on every device-side wait; 0 = 2000 ms     */
+    int32_t watchdog_ms;  /* bound on every device-side wait of the persistent
+                             engine; 0 = 2000 ms                              */
     int32_t debug_flags;  /* test hooks, 0 in normal use.  Bit 0 (persistent
                              engine): CTA 0 skips its arrival at the first
                              score barrier, so every CTA's bounded wait runs
@@ -139,7 +144,11 @@ typedef struct {
                              memory allows (at most 2048 a CTA), 1 = 256
                              entries, 2 = 1024.  0 as a whole: the shape
                              ccs_autotune recorded for this class of launch
-                             on this device, else the library's choice.   */
+                             on this device, else the library's choice.
+                             Problems that CCS_ENGINE_AUTO decodes on chip
+                             have no launch shape: a recorded one does not
+                             change them, a nonzero schedule sends them to
+                             the persistent engine.                       */
     int32_t shifted;      /* 0: Alg. 2, each column's candidate is the mode of
                              its nonzero residual values.  1: the shifted
                              variant of Sec. 4.3.1: at iteration l the only
@@ -340,11 +349,14 @@ CCS_API int ccs_decode_batch_async(const ccs_problem *probs, int32_t count,
 
 /* ---- launch-shape autotuner ---------------------------------------------------
  *
- * Not in the paper (its method fixes no launch configuration).  A batched
- * decode goes out as up to four launches, one per class of problem (d <= 8
- * or d > 8; fingerprints of r in shared memory or not).  ccs_autotune
- * decodes `probs` as ccs_decode_batch would, but runs each launch group with
- * every launch shape its kernel instances offer (CTAs of 1024, 768 or 512
+ * Not in the paper (its method fixes no launch configuration).  In the
+ * persistent engine a batched decode goes out as up to four launches, one per
+ * class of problem (d <= 8 or d > 8; fingerprints of r in shared memory or
+ * not).  ccs_autotune decodes `probs` as ccs_decode_batch does under
+ * CCS_ENGINE_PERSISTENT -- all of them, also those that CCS_ENGINE_AUTO would
+ * decode on chip: server rounds, and batches with less than a third of such
+ * problems, keep them in the persistent engine -- but runs each launch group
+ * with every launch shape its kernel instances offer (CTAs of 1024, 768 or 512
  * threads for d <= 8; 512 for d > 8; each with the CSC ring at full depth or
  * capped at 2 or 3 stages, and the candidate queue at full length or capped
  * at 256 entries: 18 shapes for d <= 8, 6 above), twice each, timing the

@@ -26,8 +26,9 @@ static size_t batch_ws(const ccs_problem *probs, int32_t count) {
     return engine_header_bytes(count) + engine_resume_header_bytes(count) + total;
 }
 
-// Time every launch shape for each launch group and record the fastest for
-// the group's class.  The shapes: the thread shapes the kernel instances
+// Time every launch shape for each launch group of the persistent engine and
+// record the fastest for the group's class (small problems among them, as a
+// server's rounds have them).  The shapes: the thread shapes the kernel instances
 // offer (d <= 8: 1024, 768 and 512 threads; d > 8: 512 only), each with
 // the CSC ring as deep as shared memory allows or capped at 2 or 3 stages,
 // and the candidate queue as long as shared memory allows or capped at 256

@@ -174,8 +174,6 @@ static int blocks_per_sm(int dev, engine_fn fn, int threads, size_t smem) {
     return per_sm;
 }
 
-// Launch the engine on P problems whose arrays are already carved out in
-// `pds` (ctrl pointers into the header of `ws`).  Fills out[0..P).
 // Launch shape of one engine launch: kernel instance, threads, shared
 // memory plan, grid.  Marks each problem's kPdUseFp flag.
 struct LaunchPlan {
@@ -352,6 +350,9 @@ static void result_of(const DecodeCtrl &c, bool timed_out, ccs_result &out) {
     out.reserved = 0;
 }
 
+// Decode P problems whose arrays are already carved out in `pds` (ctrl pointers
+// into the header of `ws`); a lone small one goes on chip.  Fills out[0..P)
+// and waits, or, with dev_out, leaves the results to the kernel.
 int engine_run(ProblemDev *pds, int P, const ccs_params &prm, ccs_result *out, char *ws,
                cudaStream_t s, ccs_result *dev_out) {
     const bool small = P == 1 && small_route(pds[0], prm, true);

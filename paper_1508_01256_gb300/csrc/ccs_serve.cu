@@ -185,7 +185,8 @@ static size_t seeded_layout(int32_t n, int32_t m, int32_t d, int32_t max_iter, i
 // Seeded requests just admitted (indices `todo` of inflight): upload each y,
 // draw each A from its seed into the pool -- every request's construction
 // enqueued first, then one wait for all their largest row degrees -- so the
-// worker waits on the stream once per admission, not once per request.  rcs[q] receives each request's status.
+// worker waits on the stream once per admission, not once per request.
+// rcs[q] receives each request's status.
 static void prepare_seeded(ccs_server *S, const std::vector<int> &todo, std::vector<int> &rcs) {
     const int Q = (int)todo.size();
     rcs.assign(Q, CCS_OK);

@@ -82,10 +82,10 @@ __device__ __forceinline__ void store_columns(const int32_t *stage, int32_t *dst
     for (int q = (ints & ~3) + threadIdx.x; q < ints; q += blockDim.x) dst[q] = stage[q];
 }
 
-// One thread a column, and one atomic add per entry counts its row.  With shift > 0 the add's result, the
-// entry's rank in its row, rides in the bits of the row index above `shift`
-// (k_place_ranked takes it out again), so that placing the transpose needs
-// no second round of atomics.
+// One thread a column, and one atomic add per entry counts its row.  With
+// shift > 0 the add's result, the entry's rank in its row, rides in the bits of
+// the row index above `shift` (k_place_ranked takes it out again), so that
+// placing the transpose needs no second round of atomics.
 //
 // Bound by the 64-bit integer work of the draws (~25 instructions each) and
 // the atomics; the entries go through shared memory so that the stores are
