@@ -325,7 +325,7 @@ CCS_API int ccs_decode_parallel_l0_async(int32_t n, int32_t m, int32_t d,
  * ccs_decode_batch -- Parallel-l0 on `count` independent problems of any
  * sizes in persistent cooperative launches (the iteration loop runs on the
  * device; each problem stops on its own rule and drops out of later
- * phases).  When a third of the problems or more are small enough for a
+ * phases).  When two fifths of the problems or more are small enough for a
  * cluster (CCS_ENGINE_AUTO), those go out in one launch of their own.  Of the
  * others, problems of one class (d <= 8 or d > 8; fingerprints of r in shared
  * memory or not) share a launch; when they are of several classes, each
@@ -354,7 +354,7 @@ CCS_API int ccs_decode_batch_async(const ccs_problem *probs, int32_t count,
  * class of problem (d <= 8 or d > 8; fingerprints of r in shared memory or
  * not).  ccs_autotune decodes `probs` as ccs_decode_batch does under
  * CCS_ENGINE_PERSISTENT -- all of them, also those that CCS_ENGINE_AUTO would
- * decode on chip: server rounds, and batches with less than a third of such
+ * decode on chip: server rounds, and batches with less than two fifths of such
  * problems, keep them in the persistent engine -- but runs each launch group
  * with every launch shape its kernel instances offer (CTAs of 1024, 768 or 512
  * threads for d <= 8; 512 for d > 8; each with the CSC ring at full depth or

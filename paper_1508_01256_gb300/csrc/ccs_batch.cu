@@ -184,16 +184,19 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
         set_last_error("at most %d problems per launch (got %d)", kMaxBatch, count);
         return CCS_EINVAL;
     }
-    // When a third of the problems or more fit a cluster on chip, those go out
-    // in one launch of the small engine.  The problems that run to max_iter
+    // When two fifths of the problems or more fit a cluster on chip, those go
+    // out in one launch of the small engine.  The problems that run to max_iter
     // decide the time of a batch: their iterations take 5-23 us there
     // against ~16 us shared by all problems in the persistent engine, which
     // has to run them anyway once one of the larger problems does not
-    // converge.  Measured, small engine against none: 39 of 44 problems fit
-    // 1.53 against 2.82 ms, 36 of 62 1.50 / 3.60, 29 of 64 2.36 / 4.51, 10 of
-    // 27 2.25 / 2.92; below a third 5 of 21 0.72 / 0.70, 7 of 41 6.57 / 6.02,
-    // 3 of 63 5.95 / 5.15.  Sending only the smaller ones of them (by n d, by
-    // m) gave the worse of both.
+    // converge.  Which problems will not is not known beforehand, so the line
+    // lies where the small engine pays on average: 66 mixed batches of 3 to 63
+    // problems, two fifths or more of them small, took 0.71 of the persistent
+    // engine's time (geometric mean; 10 took 1-43 % more, 5 of these of fewer
+    // than 20 problems).  Of 12 between a third and two fifths 5 took 7-38 %
+    // more, for 0.92 of the time on average; below, 5 of 21 small 0.72 ms
+    // against 0.70, 7 of 41 6.57 / 6.02, 3 of 63 5.95 / 5.15.  Sending only the
+    // smaller ones of them (by n d, by m) gave the worse of both.
     //
     // The others go out as up to four launches, one per class, each over the
     // whole GPU: d <= 8 and d > 8 run on different kernel instances (the
@@ -210,7 +213,7 @@ static int decode_batch_impl(const ccs_problem *probs, int32_t count, const ccs_
             ++on_chip;
         }
     for (int32_t q = 0; q < count; ++q)
-        if (cls[q] < 0 || 3 * on_chip < count)
+        if (cls[q] < 0 || 5 * on_chip < 2 * count)
             cls[q] = (pds[q].d > 8 ? 2 : 0) + (engine_fp_fits(pds[q], p) ? 0 : 1);
     // descriptors in launch order; out_slot keeps the caller's index
     std::vector<ProblemDev> sub;

@@ -159,3 +159,15 @@ def test_cluster_sizes(ccs, orc, shape, ctas):
             h = ccs.decode_batch([items, items], max_iter=30, history=True, debug_flags=flags)
             for b in h:
                 assert_same_decode(b, ref)
+
+
+@pytest.mark.parametrize("small, large", [(2, 4), (2, 3), (3, 4)])
+def test_batch_around_two_fifths(ccs, orc, small, large):
+    """From two fifths of small problems on they are decoded on chip; the
+    results are the same on both sides."""
+    probs = [inputs.make_problem(3001 + 1000 * q, 400 + 90 * q, 7, 40, 20 + q) for q in range(small)]
+    probs += [inputs.make_problem(120001 + 10000 * q, 12001, 7 + 2 * (q % 2), 900, 30 + q)
+              for q in range(large)]
+    for g, p in zip(ccs.decode_batch([device_problem(ccs, p) for p in probs], history=True), probs):
+        A, y_ref = oracle_problem(orc, p)
+        assert_same_decode(g, orc.parallel_l0(A, p.m, y_ref))
