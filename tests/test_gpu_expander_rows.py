@@ -74,8 +74,7 @@ def test_time_grows_with_the_rows(ccs):
     assert best(2 ** 29) < 8 * best(2 ** 27)
 
 
-# entries^2 / 2m, the expected pairs of entries in one row: just below one and
-# just above, and far below
+# about one expected pair of entries in a row (entries^2 / 2m), and hardly any
 @pytest.mark.parametrize("n,m,d", [(2895, 2 ** 26, 4), (2897, 2 ** 26, 4), (1003, 2 ** 26, 3)])
 def test_rows_that_most_likely_need_no_sort(ccs, orc, n, m, d):
     """Eight seeds each: some draw two columns into a row (which must come out
